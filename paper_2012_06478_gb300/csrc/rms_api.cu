@@ -7,6 +7,7 @@
 // with the same separately rounded FP64 operations as the CPU reference.
 #include <cuda_runtime.h>
 
+#include <algorithm>
 #include <atomic>
 #include <cmath>
 #include <cstdio>
@@ -49,6 +50,29 @@ __global__ void max_label_kernel(const uint16_t *lab, int64_t n, uint32_t *out)
         m = max(m, (uint32_t)lab[i]);
     for (int o = 16; o > 0; o >>= 1) m = max(m, __shfl_xor_sync(0xffffffffu, m, o));
     if ((threadIdx.x & 31) == 0) atomicMax(out, m);
+}
+
+// Face bits of every voxel (rms_device.cuh): one pass over the labels.
+__global__ void faces_kernel(const uint16_t *lab, int32_t nx, int32_t ny, int32_t nz, FastDiv div_x, FastDiv div_xy,
+                             uint8_t *faces)
+{
+    const int32_t sy = nx, sz = nx * ny;
+    const int64_t n = (int64_t)sz * nz;
+    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
+        const int32_t v = (int32_t)i;
+        const int32_t row = (int32_t)div_x.quotient((uint32_t)v), z = (int32_t)div_xy.quotient((uint32_t)v);
+        const int32_t x = v - row * nx, y = row - z * ny;
+        const uint16_t c = lab[v];
+        uint32_t f = 0u;
+        if (x > 0 && lab[v - 1] == c) f |= kFaceX;
+        if (y > 0 && lab[v - sy] == c) f |= kFaceY;
+        if (z > 0 && lab[v - sz] == c) f |= kFaceZ;
+        if (x < nx - 1 && lab[v + 1] == c) f |= kFaceX << 3;
+        if (y < ny - 1 && lab[v + sy] == c) f |= kFaceY << 3;
+        if (z < nz - 1 && lab[v + sz] == c) f |= kFaceZ << 3;
+        if (x == 0 || y == 0 || z == 0 || x == nx - 1 || y == ny - 1 || z == nz - 1) f |= kFaceEdge;
+        faces[v] = (uint8_t)f;
+    }
 }
 
 // Raster list of the voxels whose label is not dead (Sec. 2.2 item 1):
@@ -206,35 +230,21 @@ __global__ void trig_table_kernel(double *trig)
     trig[2 * j + 1] = sn;
 }
 
-// Per step: weights dt G_{s,k}, the step flags and the recording index.
-__global__ void step_tables_kernel(int64_t N, int32_t S, double dt, const double *G, const int64_t *rec,
-                                   int32_t n_rec, double *wG64, float *wG32, uint8_t *flags, int32_t *rec_of)
+// Per step: the weights dt G_{s,k} (rows of `pitch`, zeros beyond the last
+// step) and the step flags.
+__global__ void step_tables_kernel(int64_t N, int64_t pitch, int32_t S, double dt, const double *G, double *wG64,
+                                   float *wG32, uint8_t *flags)
 {
     const int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;  // 0-based step index
-    if (k >= N) return;
+    if (k >= pitch) return;
     uint8_t f = 0;
     for (int s = 0; s < S; ++s) {
-        const double w = dt * G[(int64_t)s * N + k];
-        wG64[(int64_t)s * N + k] = w;
-        wG32[(int64_t)s * N + k] = (float)w;
-        if (w != 0.0) f |= 1u;
-    }
-    // binary search of step k+1 among the recording steps
-    int lo = 0, hi = n_rec;
-    while (lo < hi) {
-        const int mid = (lo + hi) / 2;
-        if (rec[mid] < k + 1)
-            lo = mid + 1;
-        else
-            hi = mid;
-    }
-    int32_t r = -1;
-    if (lo < n_rec && rec[lo] == k + 1) {
-        r = lo;
-        f |= 2u;
+        const double w = k < N ? dt * G[(int64_t)s * N + k] : 0.0;
+        wG64[(int64_t)s * pitch + k] = w;
+        wG32[(int64_t)s * pitch + k] = (float)w;
+        if (w != 0.0) f = 1u;
     }
     flags[k] = f;
-    rec_of[k] = r;
 }
 
 __device__ __forceinline__ void neumaier(double &sum, double &comp, double x)
@@ -605,6 +615,7 @@ static rms_status upload(T **dst, const T *src, size_t n, cudaStream_t s, bool s
 static void free_substrate(rms_substrate *s, cudaStream_t st)
 {
     cudaFreeAsync(s->d_labels, st);
+    cudaFreeAsync(s->d_faces, st);
     cudaFreeAsync(s->d_D, st);
     cudaFreeAsync(s->d_T2, st);
     cudaFreeAsync(s->d_T1, st);
@@ -718,6 +729,11 @@ static rms_status create_substrate_impl(const rms_substrate_desc *d, rms_substra
     RMS_CUDA(cudaFreeAsync(d_max, st));
     RMS_CUDA(cudaStreamSynchronize(st));
     if ((int64_t)mx >= L) return fail(RMS_E_INVALID_ARG, "a label value is >= n_labels");
+    RMS_CUDA(cudaMallocAsync((void **)&s->d_faces, (size_t)nvox, st));
+    faces_kernel<<<(unsigned)std::min<int64_t>((nvox + 255) / 256, 1 << 20), 256, 0, st>>>(
+        s->d_labels, s->nx, s->ny, s->nz, FastDiv::by((uint32_t)s->nx), FastDiv::by((uint32_t)s->nx * (uint32_t)s->ny),
+        s->d_faces);
+    RMS_CUDA(cudaGetLastError());
     if (!s->conc.empty()) RMS_TRY(concentration_tables(s, nvox, st));
     bool any_dead = false;
     for (int c = 0; c < L; ++c) any_dead |= s->dead[c] != 0;
@@ -842,7 +858,7 @@ static void host_pair_tables(const rms_substrate *sub, double dt, std::vector<ui
 static void free_sequence(rms_sequence *q, cudaStream_t st)
 {
     void *p[] = {q->d_s64, q->d_dtR64, q->d_wG64, q->d_s32, q->d_dtR32, q->d_wG32, q->d_T, q->d_Tmt,
-                 q->d_flags, q->d_mode, q->d_rec_of, q->d_dirs, q->d_b, q->d_bs, q->d_q, q->d_trig};
+                 q->d_flags, q->d_mode, q->d_rec_step, q->d_dirs, q->d_b, q->d_bs, q->d_q, q->d_trig};
     for (void *x : p)
         if (x) cudaFreeAsync(x, st);
 }
@@ -884,11 +900,13 @@ static rms_status set_sequence_impl(rms_substrate *sub, const rms_sequence_desc 
     RMS_CUDA(cudaMallocAsync((void **)&q->d_dtR32, sizeof(float) * 3 * L, st));
     RMS_CUDA(cudaMallocAsync((void **)&q->d_T, sizeof(uint32_t) * (size_t)L * L, st));
     if (sub->d_rho) RMS_CUDA(cudaMallocAsync((void **)&q->d_Tmt, sizeof(uint32_t) * (size_t)L * L, st));
-    const size_t nG = (size_t)S * (N ? N : 1);
+    q->pitch = (N / 8 + 2) * 8;  // whole vectors of 8 steps, at least one step beyond the last
+    const size_t nG = (size_t)S * q->pitch;
     RMS_CUDA(cudaMallocAsync((void **)&q->d_wG64, sizeof(double) * nG, st));
     RMS_CUDA(cudaMallocAsync((void **)&q->d_wG32, sizeof(float) * nG, st));
-    RMS_CUDA(cudaMallocAsync((void **)&q->d_flags, N ? N : 1, st));
-    RMS_CUDA(cudaMallocAsync((void **)&q->d_rec_of, sizeof(int32_t) * (N ? N : 1), st));
+    RMS_CUDA(cudaMallocAsync((void **)&q->d_flags, (size_t)q->pitch, st));
+    const std::vector<int32_t> rec32(q->rec_steps.begin(), q->rec_steps.end());  // n_steps <= 2e9
+    RMS_TRY(upload(&q->d_rec_step, rec32.data(), rec32.size(), st));
     if (d->mode) {
         RMS_TRY(upload(&q->d_mode, d->mode, (size_t)N, st));
         q->has_mode = 1;
@@ -900,10 +918,8 @@ static rms_status set_sequence_impl(rms_substrate *sub, const rms_sequence_desc 
     trig_table_kernel<<<kTrigParts / 128, 128, 0, st>>>(q->d_trig);
     RMS_CUDA(cudaMallocAsync((void **)&q->d_q, sizeof(double) * S * d->n_b, st));
     double *d_G = nullptr;
-    int64_t *d_rec = nullptr;
     int32_t *d_warn = nullptr;
     RMS_TRY(upload(&d_G, d->G, (size_t)S * N, st));
-    RMS_TRY(upload(&d_rec, d->rec_steps, (size_t)d->n_rec, st));
     RMS_CUDA(cudaMallocAsync((void **)&d_warn, sizeof(int32_t), st));
     RMS_CUDA(cudaMemsetAsync(d_warn, 0, sizeof(int32_t), st));
     label_tables_kernel<<<(L + 127) / 128, 128, 0, st>>>(L, sub->d_D, sub->d_T2, sub->d_T1, d->dt_ms, sub->voxel_um,
@@ -920,17 +936,14 @@ static rms_status set_sequence_impl(rms_substrate *sub, const rms_sequence_desc 
         host_pair_tables(sub, d->dt_ms, hostT, host_warn);
         RMS_CUDA(cudaMemcpyAsync(q->d_T, hostT.data(), sizeof(uint32_t) * hostT.size(), cudaMemcpyHostToDevice, st));
     }
-    if (N > 0)
-        step_tables_kernel<<<(unsigned)((N + 255) / 256), 256, 0, st>>>(N, S, d->dt_ms, d_G, d_rec, d->n_rec,
-                                                                         q->d_wG64, q->d_wG32, q->d_flags,
-                                                                         q->d_rec_of);
+    step_tables_kernel<<<(unsigned)((q->pitch + 255) / 256), 256, 0, st>>>(N, q->pitch, S, d->dt_ms, d_G, q->d_wG64,
+                                                                            q->d_wG32, q->d_flags);
     bvalue_kernel<<<(unsigned)std::max(S, 1), kBvThreads, 0, st>>>(N, S, d->dt_ms, d_G, d->n_b, q->d_b, q->d_bs,
                                                                     q->d_q);
     RMS_CUDA(cudaGetLastError());
     int32_t w = 0;
     RMS_CUDA(cudaMemcpyAsync(&w, d_warn, sizeof(int32_t), cudaMemcpyDeviceToHost, st));
     RMS_CUDA(cudaFreeAsync(d_G, st));
-    RMS_CUDA(cudaFreeAsync(d_rec, st));
     RMS_CUDA(cudaFreeAsync(d_warn, st));
     RMS_CUDA(cudaStreamSynchronize(st));
     *warn = w != 0 || host_warn;
@@ -1020,15 +1033,17 @@ ReqDesc<Real> rms::run_desc(rms_run_handle *r)
     rms_sequence *q = r->seq;
     rms_substrate *sub = q->sub;
     ReqDesc<Real> d{};
-    d.g = Geometry{sub->d_labels, sub->nx, sub->ny, sub->nz, sub->periodic[0], sub->periodic[1], sub->periodic[2],
-                   sub->voxel_um, (float)sub->voxel_um};
+    d.g = Geometry{sub->d_labels, sub->d_faces, FastDiv::by((uint32_t)sub->nx),
+                   FastDiv::by((uint32_t)sub->nx * (uint32_t)sub->ny), sub->nx, sub->ny, sub->nz,
+                   sub->periodic[0] | sub->periodic[1] << 1 | sub->periodic[2] << 2, sub->voxel_um,
+                   (float)sub->voxel_um};
     if constexpr (std::is_same<Real, float>::value) {
-        d.t = Tables<float>{q->d_s32, q->d_dtR32, q->d_T, q->d_Tmt, sub->L, q->d_wG32, q->d_flags, q->d_rec_of,
-                            q->d_mode, q->any_relax, q->d_trig};
+        d.t = Tables<float>{q->d_s32, q->d_dtR32, q->d_T, q->d_Tmt, sub->L, q->d_wG32, q->pitch, q->d_flags,
+                            q->d_rec_step, q->d_mode, q->any_relax, q->d_trig};
         d.st = r->st32;
     } else {
-        d.t = Tables<double>{q->d_s64, q->d_dtR64, q->d_T, q->d_Tmt, sub->L, q->d_wG64, q->d_flags, q->d_rec_of,
-                             q->d_mode, q->any_relax, q->d_trig};
+        d.t = Tables<double>{q->d_s64, q->d_dtR64, q->d_T, q->d_Tmt, sub->L, q->d_wG64, q->pitch, q->d_flags,
+                             q->d_rec_step, q->d_mode, q->any_relax, q->d_trig};
         d.st = r->st64;
     }
     d.ctl.seed = r->seed;
@@ -1071,8 +1086,9 @@ static rms_status walk_impl(rms_run_handle *r, int64_t k0, int64_t k1)
     const bool hash = (r->flags & kVerifyFlags) != 0;  // the verification kernel
     const dim3 grid((unsigned)r->n_blocks);
     const int S = r->seq->S;
+    const int32_t rec = first_rec(r->seq, k0);
 #define RMS_WALK(IM, MT) \
-    RMS_CUDA((launch_walk<Real, IM, MT>(S, hash, grid, r->stream, d.g, d.t, d.st, d.ctl, k0, k1)))
+    RMS_CUDA((launch_walk<Real, IM, MT>(S, hash, grid, r->stream, d.g, d.t, d.st, d.ctl, k0, k1, rec)))
     const bool mt = d.t.Tmt != nullptr;
     switch (r->interaction) {
     case RMS_RS:

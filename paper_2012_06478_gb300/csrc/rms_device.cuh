@@ -143,10 +143,35 @@ struct WalkerState {
     int32_t *wid;      // walker (relative to the run's first) in each slot, or nullptr: the slot's index
 };
 
+// Quotients n / d for 0 <= n < 2^31 by a multiplication: with 2^(l-1) < d <=
+// 2^l, mul = ceil(2^(31+l) / d) < 2^32 and n mul >> (31 + l) is the quotient,
+// since the excess mul d - 2^(31+l) < 2^l adds less than n 2^l < 2^(31+l) to
+// n 2^(31+l) / d (Granlund & Montgomery 1994).
+struct FastDiv {
+    uint32_t mul, shift;
+    __host__ __device__ uint32_t quotient(uint32_t n) const { return (uint32_t)(((uint64_t)n * mul) >> shift); }
+    static FastDiv by(uint32_t d)
+    {
+        uint32_t l = 0;
+        while ((1ull << l) < d) ++l;
+        return FastDiv{(uint32_t)((((uint64_t)1 << (31 + l)) + d - 1) / d), 31 + l};
+    }
+};
+
+// Face bits of a voxel: per axis, that the voxel across its lower (bits 0-2)
+// or upper face (bits 3-5) lies inside the volume and carries the same label;
+// and that the voxel touches the volume's outer faces.  Most face events
+// stay inside a label (Sec. 2.1.1: the label volume is its own lookup table),
+// and a byte per voxel decides them: half the label volume's bytes, read
+// ahead of the event that needs them.
+enum : uint32_t { kFaceX = 1u, kFaceY = 2u, kFaceZ = 4u, kFaceEdge = 64u };
+
 struct Geometry {
     const uint16_t *labels;
+    const uint8_t *faces;  // face bits per voxel
+    FastDiv div_x, div_xy; // by nx and nx ny
     int32_t nx, ny, nz;
-    int32_t per_x, per_y, per_z;
+    int32_t periodic;      // bit a: axis a is periodic
     double voxel_um;
     float voxel_f;  // voxel_um rounded to single precision (the FP32 form's phase)
 };
@@ -158,9 +183,10 @@ struct Tables {
     const uint32_t *T;      // [from][to] Bernoulli thresholds
     const uint32_t *Tmt;    // [from][to] saturation thresholds (MT), or nullptr
     int32_t n_labels;
-    const Real *wG;         // [shape][step]: dt * G
-    const uint8_t *flags;   // [step]: bit0 any G != 0, bit1 recording step
-    const int32_t *rec_of;  // [step]: recording index or -1
+    const Real *wG;         // [shape][pitch]: dt * G of each step, zeros beyond the last
+    int64_t pitch;
+    const uint8_t *flags;   // [step]: 1 where some shape's G != 0
+    const int32_t *rec_step;  // [n_rec] recording steps
     const uint8_t *mode;    // [step] relaxation mode (or nullptr = 0)
     int32_t any_relax;
     const double *trig;     // [part][cos, sin] of the azimuth table (FP64 form)
@@ -191,9 +217,10 @@ struct ReqDesc {
 };
 
 // One block of a batched launch: block `block` of request `req`, steps (k0, k1].
+// `rec`: the first recording step's index beyond k0.
 struct BlockTask {
     int32_t req;
-    int32_t pad;
+    int32_t rec;
     int64_t block;
     int64_t k0, k1;
 };

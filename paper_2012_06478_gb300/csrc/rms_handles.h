@@ -4,6 +4,7 @@
 
 #include <cuda_runtime.h>
 
+#include <algorithm>
 #include <atomic>
 #include <string>
 #include <vector>
@@ -36,6 +37,7 @@ struct rms_substrate {
     uint64_t *d_acc = nullptr;  // per label start acceptance threshold (nullptr: always)
     std::vector<uint8_t> dead;
     uint16_t *d_labels = nullptr;
+    uint8_t *d_faces = nullptr;  // face bits per voxel (rms_device.cuh)
     double *d_D = nullptr, *d_T2 = nullptr, *d_T1 = nullptr, *d_kappa = nullptr, *d_rho = nullptr;
     uint8_t *d_dead = nullptr;
     int32_t *d_ok = nullptr;  // raster list of non-dead voxels (nullptr: none dead)
@@ -56,7 +58,8 @@ struct rms_sequence {
     uint32_t *d_T = nullptr;
     uint32_t *d_Tmt = nullptr;  // saturation thresholds (nullptr: no absorbing membrane)
     uint8_t *d_flags = nullptr, *d_mode = nullptr;
-    int32_t *d_rec_of = nullptr;
+    int32_t *d_rec_step = nullptr;
+    int64_t pitch = 0;  // row pitch of d_wG64 and d_wG32
     double *d_dirs = nullptr, *d_b = nullptr, *d_bs = nullptr, *d_q = nullptr;
     double *d_trig = nullptr;  // azimuth table (FP64 form)
     std::atomic<int> refs{0};
@@ -111,6 +114,12 @@ rms_status fail(rms_status st, const std::string &msg);
         rms_status st_ = (expr); \
         if (st_ < 0) return st_; \
     } while (0)
+
+// The index of the first recording step beyond step k0.
+inline int32_t first_rec(const rms_sequence *q, int64_t k0)
+{
+    return (int32_t)(std::upper_bound(q->rec_steps.begin(), q->rec_steps.end(), k0) - q->rec_steps.begin());
+}
 
 // The normalised signal [combo][2] + (alpha sum, 0) of a finalised run.
 inline double *normalised_S(const rms_run_handle *r) { return r->d_S + 2 * (size_t)(r->n_combo + 1); }

@@ -10,12 +10,12 @@ namespace rms {
 template <typename Real, int IM, bool MT>
 cudaError_t launch_walk(int n_shapes, bool hash, dim3 grid, cudaStream_t stream, const Geometry &g,
                         const Tables<Real> &t, const WalkerState<Real> &st, const RunCtl &ctl,
-                        int64_t k_begin, int64_t k_end);
+                        int64_t k_begin, int64_t k_end, int32_t rec);
 
 #define RMS_EXTERN_LAUNCH_WALK(REAL, IM, MT)                                                               \
     extern template cudaError_t launch_walk<REAL, IM, MT>(int, bool, dim3, cudaStream_t, const Geometry &, \
                                                           const Tables<REAL> &, const WalkerState<REAL> &, \
-                                                          const RunCtl &, int64_t, int64_t);
+                                                          const RunCtl &, int64_t, int64_t, int32_t);
 RMS_EXTERN_LAUNCH_WALK(double, kInteractEC, false)
 RMS_EXTERN_LAUNCH_WALK(double, kInteractRS, false)
 RMS_EXTERN_LAUNCH_WALK(double, kInteractERL, false)

@@ -300,7 +300,8 @@ rms_status tick_once(rms_server *s)
                 const int64_t k1 = std::min<int64_t>(q->seq->n_steps, k0 + quota);
                 range[i] = {k0, k1};
                 ++q->ticks;
-                for (int64_t b = 0; b < q->run->n_blocks; ++b) T[off++] = BlockTask{q->slot, 0, b, k0, k1};
+                const int32_t rec = first_rec(q->seq, k0);
+                for (int64_t b = 0; b < q->run->n_blocks; ++b) T[off++] = BlockTask{q->slot, rec, b, k0, k1};
             }
         count[g] = off - start[g];
     }

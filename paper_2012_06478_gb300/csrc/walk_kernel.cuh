@@ -9,10 +9,18 @@
 // One thread owns one walker for a slice of steps; its whole state stays in
 // registers for the slice and goes back to global memory (structure of
 // arrays, coalesced) at the end.  Per step and walker the only memory
-// traffic is the dependent 2-byte label gather across each face met
-// (Sec. 2.1.1: the label volume is the lookup table), the threshold of the
-// label pair at a membrane (and its saturation threshold, with absorbing
+// traffic is one byte for each voxel entered -- its face bits, which say
+// whether each of the voxel's faces leads into the same label (Sec. 2.1.1: the
+// volume is the lookup table) -- at a membrane the label across it and the
+// threshold of the label pair (and its saturation threshold, with absorbing
 // membranes), and warp-uniform broadcasts of the waveform.
+//
+// What bounds it: the FP32 step issues (323 warp-instructions per warp-step on
+// 200x200x400 axons, issue slots 74 % used, ALU pipe 65 %).  Deciding the
+// events from face bits instead of a label gather with wrapped coordinates,
+// with selects in place of branches, the step's tables and weights read ahead
+// and nothing done for relaxation when no label relaxes took 1e6 walkers x
+// 2000 steps from 27.4 ms (428 warp-instructions) to 21.8 ms, the same bits.
 #pragma once
 
 #include <cstdint>
@@ -184,6 +192,23 @@ __device__ __forceinline__ void direction_from(uint32_t x0, uint32_t x1, const d
     n[2] = z;
 }
 
+// a / b for b > 0 as a times the hardware reciprocal (its error is within 1 ulp),
+// infinite for b = 0 -- the bits of __fdividef for every normal b, without its
+// rescaling of subnormal divisors: the FP32 step's divisors |d| are zero or
+// above 1e-13 of the step length.  Likewise the reciprocal square root.
+__device__ __forceinline__ float mul_rcp(float a, float b)
+{
+    float r;
+    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(b));
+    return a * r;
+}
+__device__ __forceinline__ float rsqrt_normal(float x)
+{
+    float r;
+    asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
+    return r;
+}
+
 // FP32 form of the same sampler: shorter polynomials (truncation below
 // 4e-7 on [0, pi/4]) and r from the hardware reciprocal square root (about
 // 2 ulp; (1 - z)(1 + z) > 0 since |z| < 1) -- errors of the order of the FP32
@@ -192,7 +217,7 @@ __device__ __forceinline__ void direction_from(uint32_t x0, uint32_t x1, const d
 {
     const float z = -((float)(int32_t)(x0 ^ 0x80000000u) + 0.5f) * 0x1p-31f;
     const float rr = (1.0f - z) * (1.0f + z);
-    const float r = rr * rsqrtf(rr);
+    const float r = rr * rsqrt_normal(rr);
     const uint32_t oct = x1 >> 29;
     uint32_t m = x1 & 0x1FFFFFFFu;
     if (oct & 1u) m = 0x1FFFFFFFu - m;
@@ -226,6 +251,31 @@ __device__ __forceinline__ void saturate(float &A, float &Ac)
 static __device__ __noinline__ uint32_t perm_word(uint64_t seed, uint64_t w, uint32_t k, uint32_t call)
 {
     return draw(seed, w, k, kTagPerm, call).x;
+}
+
+// Coordinate q modulo N, in [0, N).
+__device__ __forceinline__ int32_t wrapped(int32_t q, int32_t N)
+{
+    q %= N;
+    return q < 0 ? q + N : q;
+}
+
+// A face event of an edge voxel v: the voxel across -- nv, or the one on the
+// periodic other side -- or -1 for the impermeable outer wall.  The
+// coordinates come from the flat index by multiplication (no division).  Out
+// of line, on values: a few events in a thousand on volumes of a hundred
+// voxels an edge.
+static __device__ __noinline__ int32_t edge_voxel(int32_t v, int32_t nv, int best, bool up, int32_t nx, int32_t ny,
+                                                  int32_t nz, FastDiv div_x, FastDiv div_xy, int32_t periodic)
+{
+    const int32_t row = (int32_t)div_x.quotient((uint32_t)v);    // v / nx
+    const int32_t z = (int32_t)div_xy.quotient((uint32_t)v);     // v / (nx ny)
+    const int32_t coord = best == 2 ? z : (best == 1 ? row - z * ny : v - row * nx);
+    const int32_t N = best == 2 ? nz : (best == 1 ? ny : nx);
+    if (coord != (up ? N - 1 : 0)) return nv;
+    if (!((periodic >> best) & 1)) return -1;
+    const int32_t sb = best == 2 ? nx * ny : (best == 1 ? nx : 1);
+    return up ? v - (N - 1) * sb : v + (N - 1) * sb;
 }
 
 __device__ __forceinline__ double warp_sum(double v)
@@ -285,13 +335,17 @@ __device__ __forceinline__ void warp_moments(double al, const double dx[3], doub
 // it was for the step, ERL draws a new direction (DIR and PERM call = the
 // draw's index) until a step is admitted, at most kMaxLeaps draws.  MT adds
 // absorbing membranes (Sec. 2.1.3, magnetization transfer; t.Tmt non-null).
+// RELAX: 1 some label has a finite T1 or T2, 0 none has (every rate is 0, the
+// exponent keeps its start value and Eq. 5 drops out), 2 decided at run time.
 // RK: draw with the round keys of ctl.rk, computed once on the host (no key
 // schedule per draw: 2.4 % faster on the FP32 step); otherwise advance the
 // key from ctl.seed in every draw (the batched kernel, whose request
-// descriptors sit in shared memory).
-template <typename Real, int NS, bool HASH, int IM, bool MT, bool RK = false>
+// descriptors sit in shared memory).  `rec` is the first recording step's
+// index beyond k_begin.
+template <typename Real, int NS, bool HASH, int IM, bool MT, int RELAX, bool RK = false>
 __device__ __forceinline__ void walk_block(const Geometry &g, const Tables<Real> &t, const WalkerState<Real> &st,
-                                           const RunCtl &ctl, int64_t block, int64_t k_begin, int64_t k_end)
+                                           const RunCtl &ctl, int64_t block, int64_t k_begin, int64_t k_end,
+                                           int32_t rec)
 {
     constexpr bool kF64 = std::is_same<Real, double>::value;
     __shared__ int32_t s_cancel;
@@ -306,15 +360,17 @@ __device__ __forceinline__ void walk_block(const Geometry &g, const Tables<Real>
     uint32_t rk[kRoundKeys];
 #pragma unroll
     for (int i = 0; i < kRoundKeys; ++i) rk[i] = ctl.rk[i];
-    const int64_t li = block * kWalkBlock + threadIdx.x;
-    const bool active = li < ctl.n_walkers;
+    // threads beyond the last walker walk a copy of it and write nothing: no
+    // branch on it in the step loop
+    const bool active = block * kWalkBlock + threadIdx.x < ctl.n_walkers;
+    const int64_t li = active ? block * kWalkBlock + threadIdx.x : ctl.n_walkers - 1;
     // the walker in this slot: its id picks its random streams (RMS_MORTON
     // runs keep walkers in Morton order of their voxel, not in id order)
-    const uint64_t w = (uint64_t)(ctl.w_begin + ((active && st.wid) ? (int64_t)st.wid[li] : li));
+    const uint64_t w = (uint64_t)(ctl.w_begin + (st.wid ? (int64_t)st.wid[li] : li));
     const int32_t N[3] = {g.nx, g.ny, g.nz};
     const int32_t stride[3] = {1, g.nx, g.nx * g.ny};
-    const int32_t per[3] = {g.per_x, g.per_y, g.per_z};
     const int32_t L = t.n_labels;
+    const bool relax = RELAX == 2 ? t.any_relax != 0 : RELAX == 1;
     // voxel edge in the form's precision (the single-precision value comes from
     // the host: a conversion here would run on the FP64 pipe at every step)
     Real lp;
@@ -324,85 +380,84 @@ __device__ __forceinline__ void walk_block(const Geometry &g, const Tables<Real>
         lp = g.voxel_f;
 
     Real o[3], o0[3];
-    int32_t di[3], wc[3];
-    int32_t v = 0, c = 0;
-    Real A = Real(0), Ac = Real(0);
+    int32_t di[3];
+    int32_t v = 0;
+#pragma unroll
+    for (int a = 0; a < 3; ++a) {
+        o[a] = st.o[a][li];
+        o0[a] = st.o0[a][li];
+        di[a] = st.di[a][li];
+        v += stride[a] * wrapped(st.i0[a][li] + di[a], N[a]);
+    }
+    uint32_t fm = __ldg(g.faces + v);  // face bits of voxel v (rms_device.cuh)
+    int32_t c = st.c[li];
+    Real sc = __ldg(t.s + c);  // step length of label c
+    Real A = st.A[li], Ac = Real(0);
+    if constexpr (!kF64) Ac = st.A_c[li];
     Real ph[NS][3], phc[NS][3];
-    uint64_t h = 0;
+#pragma unroll
+    for (int s = 0; s < NS; ++s)
+#pragma unroll
+        for (int a = 0; a < 3; ++a) {
+            ph[s][a] = s < ctl.n_shapes ? st.phase[((int64_t)s * 3 + a) * ctl.n_walkers + li] : Real(0);
+            phc[s][a] =
+                (!kF64 && s < ctl.n_shapes) ? st.phase_c[((int64_t)s * 3 + a) * ctl.n_walkers + li] : Real(0);
+        }
+    [[maybe_unused]] uint64_t h = 0;
     // face events, crossings into another label, reflections (verification kernel)
     [[maybe_unused]] int32_t nev = 0, ncr = 0, nrf = 0;
-    if (active) {
-#pragma unroll
-        for (int a = 0; a < 3; ++a) {
-            o[a] = st.o[a][li];
-            o0[a] = st.o0[a][li];
-            di[a] = st.di[a][li];
-            int32_t q = (st.i0[a][li] + di[a]) % N[a];
-            wc[a] = q < 0 ? q + N[a] : q;
+    if constexpr (HASH) {
+        h = st.hash[li];
+        if (st.counts) {
+            nev = st.counts[li];
+            ncr = st.counts[ctl.n_walkers + li];
+            nrf = st.counts[2 * ctl.n_walkers + li];
         }
-        v = wc[0] + stride[1] * wc[1] + stride[2] * wc[2];
-        c = st.c[li];
-        A = st.A[li];
-        if (!kF64) Ac = st.A_c[li];
-#pragma unroll
-        for (int s = 0; s < NS; ++s)
-#pragma unroll
-            for (int a = 0; a < 3; ++a) {
-                ph[s][a] = s < ctl.n_shapes ? st.phase[((int64_t)s * 3 + a) * ctl.n_walkers + li] : Real(0);
-                phc[s][a] = (!kF64 && s < ctl.n_shapes)
-                                ? st.phase_c[((int64_t)s * 3 + a) * ctl.n_walkers + li]
-                                : Real(0);
-            }
-        if (HASH) h = st.hash[li];
-        if constexpr (HASH) {
-            if (st.counts) {
-                nev = st.counts[li];
-                ncr = st.counts[ctl.n_walkers + li];
-                nrf = st.counts[2 * ctl.n_walkers + li];
-            }
-        }
-    } else {
-#pragma unroll
-        for (int a = 0; a < 3; ++a) {
-            o[a] = o0[a] = Real(0);
-            di[a] = wc[a] = 0;
-        }
-#pragma unroll
-        for (int s = 0; s < NS; ++s)
-#pragma unroll
-            for (int a = 0; a < 3; ++a) ph[s][a] = phc[s][a] = Real(0);
     }
+    int32_t next_rec = rec < ctl.n_rec ? __ldg(t.rec_step + rec) : INT32_MAX;
 
     // a 32-bit step counter (n_steps <= 2e9): uniform 32-bit arithmetic per
     // step (measured 0.8 % faster than 64-bit on the FP32 step)
     for (int32_t k = (int32_t)k_begin + 1; k <= (int32_t)k_end; ++k) {
-        const uint8_t fl = __ldg(t.flags + (k - 1));
-        if (active) {
-            const int mode = t.mode ? (int)__ldg(t.mode + (k - 1)) : 0;
-            // state at the step start, restored when a membrane refuses the step
-            [[maybe_unused]] Real o_s[3], A_s, Ac_s;
-            [[maybe_unused]] int32_t wc_s[3], di_s[3], v_s, c_s, nev_s, ncr_s, nrf_s;
-            if constexpr (IM != kInteractEC) {
+        // the step's weight dt G_k, asked for before the walk (several shapes: a flag
+        // that one of them is not zero)
+        [[maybe_unused]] Real wg = Real(0);
+        bool graded;
+        if constexpr (NS == 1) {
+            wg = __ldg(t.wG + (k - 1));
+            graded = wg != Real(0);
+        } else {
+            graded = (__ldg(t.flags + (k - 1)) & 1u) != 0u;
+        }
+        int mode = 0;
+        if (relax) mode = t.mode ? (int)__ldg(t.mode + (k - 1)) : 0;
+        // state at the step start, restored when a membrane refuses the step
+        [[maybe_unused]] Real o_s[3], A_s, Ac_s;
+        [[maybe_unused]] int32_t di_s[3], v_s, c_s, nev_s, ncr_s, nrf_s;
+        [[maybe_unused]] uint32_t fm_s;
+        [[maybe_unused]] Real sc_s;
+        if constexpr (IM != kInteractEC) {
 #pragma unroll
-                for (int a = 0; a < 3; ++a) {
-                    o_s[a] = o[a];
-                    wc_s[a] = wc[a];
-                    di_s[a] = di[a];
-                }
-                v_s = v;
-                c_s = c;
-                A_s = A;
-                Ac_s = Ac;
-                if constexpr (HASH) {
-                    nev_s = nev;
-                    ncr_s = ncr;
-                    nrf_s = nrf;
-                }
+            for (int a = 0; a < 3; ++a) {
+                o_s[a] = o[a];
+                di_s[a] = di[a];
             }
-            uint32_t att = 0;  // draw index (ERL redraws); always 0 otherwise
-            [[maybe_unused]] bool sat_any = false;  // saturated on some draw of this step (MT)
+            v_s = v;
+            fm_s = fm;
+            c_s = c;
+            sc_s = sc;
+            A_s = A;
+            Ac_s = Ac;
+            if constexpr (HASH) {
+                nev_s = nev;
+                ncr_s = ncr;
+                nrf_s = nrf;
+            }
+        }
+        uint32_t att = 0;  // draw index (ERL redraws); always 0 otherwise
+        [[maybe_unused]] bool sat_any = false;  // saturated on some draw of this step (MT)
 #pragma unroll 1
-            for (;;) {
+        for (;;) {
             // ---- direction (one DIR call: words 0, 1 -> direction; words 2, 3 ->
             //      the Bernoulli words of the step's first two membrane events)
             U4 x;
@@ -413,43 +468,21 @@ __device__ __forceinline__ void walk_block(const Geometry &g, const Tables<Real>
             Real n[3];
             direction_from(x.x, x.y, t.trig, n);
             // ---- face walk (Sec. 2.2 items 3-4)
-            Real sc = __ldg(t.s + c);
-            Real rate = t.any_relax ? __ldg(t.dtR + mode * L + c) : Real(0);
+            Real rate = Real(0);
+            if (relax) rate = __ldg(t.dtR + mode * L + c);
             [[maybe_unused]] const Real rate0 = rate;
             Real d[3] = {mulr(n[0], sc), mulr(n[1], sc), mulr(n[2], sc)};
             [[maybe_unused]] bool refused = false;
-            // A face event on axis `best` moving up/down: look up the voxel across
-            // it and decide between crossing and reflection.
-            auto face = [&](int best, bool up, int ev) -> bool {
-                int32_t coord = 0, Nb = 1, sb = 1, pb = 1;
-#pragma unroll
-                for (int a = 0; a < 3; ++a)
-                    if (a == best) {
-                        coord = wc[a];
-                        Nb = N[a];
-                        sb = stride[a];
-                        pb = per[a];
-                    }
-                int32_t nc, nv;
-                bool wall = false;
-                if (up) {
-                    nc = coord + 1;
-                    nv = v + sb;
-                    if (nc == Nb) {
-                        wall = !pb;
-                        nc = 0;
-                        nv = v - (Nb - 1) * sb;
-                    }
-                } else {
-                    nc = coord - 1;
-                    nv = v - sb;
-                    if (coord == 0) {
-                        wall = !pb;
-                        nc = Nb - 1;
-                        nv = v + (Nb - 1) * sb;
-                    }
-                }
-                const int32_t c2 = wall ? -1 : (int32_t)__ldg(g.labels + nv);
+            // A face event on axis `best` moving up/down: where the voxel's own face
+            // bits say that the voxel across is inside the volume and carries the same
+            // label -- nearly every event -- nothing is looked up to decide it: the
+            // walker moves on, and the new voxel's bits, which the next event needs,
+            // load meanwhile.  membrane() takes any other face: nv becomes the voxel
+            // across; true when the walker crosses (changed: into another label).
+            auto membrane = [&](int best, bool up, int ev, int32_t &nv, bool &changed) -> bool {
+                if (fm & kFaceEdge)
+                    nv = edge_voxel(v, nv, best, up, g.nx, g.ny, g.nz, g.div_x, g.div_xy, g.periodic);
+                const int32_t c2 = nv < 0 ? -1 : (int32_t)__ldg(g.labels + nv);
                 // magnetization transfer (Sec. 2.1.3): meeting an absorbing membrane
                 // saturates the walker with probability P_MT -- word `ev` of the
                 // step's MT call (call = the draw index)
@@ -462,38 +495,23 @@ __device__ __forceinline__ void walk_block(const Geometry &g, const Tables<Real>
                         }
                     }
                 }
-                bool cross;
-                if (c2 == c) {
-                    cross = true;
-                } else if (c2 < 0) {
-                    cross = false;
-                } else {
-                    const uint32_t T = __ldg(t.T + (int64_t)c * L + c2);
-                    if (T == 0u) {
-                        cross = false;
-                    } else {
-                        // third membrane event of a step: word 0 of the step's PERM call
-                        const uint32_t word =
-                            ev == 0 ? x.z : (ev == 1 ? x.w : perm_word(ctl.seed, w, (uint32_t)k, att));
-                        cross = word < T;
-                    }
+                if (c2 == c) return true;
+                const uint32_t T = c2 < 0 ? 0u : __ldg(t.T + (int64_t)c * L + c2);
+                bool cross = false;
+                if (T != 0u) {
+                    // third membrane event of a step: word 0 of the step's PERM call
+                    const uint32_t word =
+                        ev == 0 ? x.z : (ev == 1 ? x.w : perm_word(ctl.seed, w, (uint32_t)k, att));
+                    cross = word < T;
                 }
                 if (cross) {
-#pragma unroll
-                    for (int a = 0; a < 3; ++a)
-                        if (a == best) {
-                            wc[a] = nc;
-                            di[a] += up ? 1 : -1;
-                            o[a] = up ? Real(0) : Real(1);
-                        }
-                    v = nv;
-                    if (c2 != c) {
-                        if constexpr (HASH) ++ncr;
-                        c = c2;
-                        if (t.any_relax) rate = __ldg(t.dtR + mode * L + c);
-                        return true;  // the caller switches to the new label's step length
-                    }
-                } else if constexpr (IM != kInteractEC) {
+                    if constexpr (HASH) ++ncr;
+                    c = c2;
+                    if (relax) rate = __ldg(t.dtR + mode * L + c);
+                    changed = true;  // the caller switches to the new label's step length
+                    return true;
+                }
+                if constexpr (IM != kInteractEC) {
                     refused = true;
                 } else {
                     if constexpr (HASH) ++nrf;
@@ -544,107 +562,136 @@ __device__ __forceinline__ void walk_block(const Geometry &g, const Tables<Real>
                     }
                     if (!dlt_nn(tmin, 1.0)) break;
                     const double dts = tmin - tau;
+                    if (relax) A = A + dmul(dts, rate);
+                    tau = tmin;
+                    if constexpr (HASH) ++nev;
                     bool up = false;
 #pragma unroll
                     for (int a = 0; a < 3; ++a) {
                         if (a == best) {
                             up = dgt0(d[a]);
-                            o[a] = up ? 1.0 : 0.0;
                             T[a] = kInf;
+                            o[a] = up ? 0.0 : 1.0;
+                            di[a] += up ? 1 : -1;
                         } else {
                             o[a] = dclamp01(o[a] + dmul(dts, d[a]));
                         }
                     }
-                    if (t.any_relax) A = A + dmul(dts, rate);
-                    tau = tmin;
-                    if constexpr (HASH) ++nev;
-                    const bool changed = face(best, up, ev);
-                    if constexpr (IM != kInteractEC) {
-                        if (refused) break;
-                    }
-                    if (changed) {
-                        const double sn = __ldg(t.s + c);
-                        if (dbits(sn) != dbits(sc)) {
-                            sc = sn;
+                    const int32_t sb = best == 2 ? stride[2] : (best == 1 ? stride[1] : 1);
+                    const uint32_t bit = (best == 2 ? kFaceZ : (best == 1 ? kFaceY : kFaceX)) << (up ? 3 : 0);
+                    int32_t nv = up ? v + sb : v - sb;
+                    if (!(fm & bit)) {
+                        bool changed = false;
+                        if (!membrane(best, up, ev, nv, changed)) {  // stays in its voxel, at the face
+                            nv = v;
 #pragma unroll
-                            for (int a = 0; a < 3; ++a) {
-                                d[a] = dmul(n[a], sc);
-                                if (dbits(T[a]) == 0x7FF0000000000000LL) continue;
-                                const double num = dgt0(d[a]) ? 1.0 - o[a] : o[a];
-                                T[a] = tau + ddiv_nn(num, __longlong_as_double(dbits(d[a]) & 0x7FFFFFFFFFFFFFFFLL));
+                            for (int a = 0; a < 3; ++a)
+                                if (a == best) {
+                                    o[a] = up ? 1.0 : 0.0;
+                                    di[a] -= up ? 1 : -1;
+                                }
+                        }
+                        if (changed) {
+                            const double sn = __ldg(t.s + c);
+                            if (dbits(sn) != dbits(sc)) {
+                                sc = sn;
+#pragma unroll
+                                for (int a = 0; a < 3; ++a) {
+                                    d[a] = dmul(n[a], sc);
+                                    if (dbits(T[a]) == 0x7FF0000000000000LL) continue;
+                                    const double num = dgt0(d[a]) ? 1.0 - o[a] : o[a];
+                                    T[a] = tau +
+                                           ddiv_nn(num, __longlong_as_double(dbits(d[a]) & 0x7FFFFFFFFFFFFFFFLL));
+                                }
                             }
                         }
+                    }
+                    v = nv;
+                    fm = __ldg(g.faces + v);
+                    if constexpr (IM != kInteractEC) {
+                        if (refused) break;
                     }
                 }
                 if (IM == kInteractEC || !refused) {
                     const double rem = 1.0 - tau;
 #pragma unroll
                     for (int a = 0; a < 3; ++a) o[a] = dclamp01(o[a] + dmul(rem, d[a]));
-                    if (t.any_relax) A = A + dmul(rem, rate);
+                    if (relax) A = A + dmul(rem, rate);
                 }
             } else {
-                // Precision form: the same walk in FP32 (approximate division).
+                // Precision form: the same walk in FP32.  The choices are selects and
+                // predicated instructions; only the end test and the membrane branch, and a
+                // membrane that is not crossed takes back the crossing assumed before it.
                 constexpr Real kNever = Real(1e30);
                 Real T[3];
 #pragma unroll
                 for (int a = 0; a < 3; ++a) {
-                    const Real ad = fabsf(d[a]);
-                    const Real dist = d[a] > Real(0) ? Real(1) - o[a] : o[a];
-                    T[a] = ad > Real(0) ? fminf(__fdividef(dist, ad), kNever) : kNever;
+                    const bool up = d[a] > Real(0);
+                    T[a] = fminf(mul_rcp(up ? Real(1) - o[a] : o[a], fabsf(d[a])), kNever);
                 }
                 Real tau = Real(0);
 #pragma unroll  // unrolled: each event index is a constant (measured 5 % faster, FP32)
                 for (int ev = 0; ev < 3; ++ev) {
-                    int best = 0;
-                    Real tmin = T[0];
-                    if (T[1] < tmin) {
-                        best = 1;
-                        tmin = T[1];
-                    }
-                    if (T[2] < tmin) {
-                        best = 2;
-                        tmin = T[2];
-                    }
+                    const bool b1 = T[1] < T[0];
+                    const Real t01 = fminf(T[0], T[1]);
+                    const bool b2 = T[2] < t01;
+                    Real tmin = fminf(t01, T[2]);
                     if (!(tmin < Real(1))) break;
-                    tmin = fmaxf(tmin, tau);
-                    const Real dtt = tmin - tau;
-                    bool up = false;
-#pragma unroll
-                    for (int a = 0; a < 3; ++a) {
-                        if (a == best) {
-                            up = d[a] > Real(0);
-                            o[a] = up ? Real(1) : Real(0);
-                            T[a] = kNever;
-                        } else {
-                            o[a] = clamp01(o[a] + dtt * d[a]);
-                        }
-                    }
-                    if (t.any_relax) kahan_add(A, Ac, dtt * rate);
+                    if (ev > 0) tmin = fmaxf(tmin, tau);
+                    const Real dtt = ev > 0 ? tmin - tau : tmin;
+                    if (relax) kahan_add(A, Ac, dtt * rate);
                     tau = tmin;
                     if constexpr (HASH) ++nev;
-                    const bool changed = face(best, up, ev);
-                    if constexpr (IM != kInteractEC) {
-                        if (refused) break;
-                    }
-                    if (changed) {
-                        const Real sn = __ldg(t.s + c);
-                        if (sn != sc) {
-                            sc = sn;
+                    const int best = b2 ? 2 : (b1 ? 1 : 0);
+                    const bool up = (b2 ? d[2] : (b1 ? d[1] : d[0])) > Real(0);
+                    const int32_t sb = b2 ? stride[2] : (b1 ? stride[1] : 1);
+                    int32_t nv = up ? v + sb : v - sb;
+                    const uint32_t bit = (b2 ? kFaceZ : (b1 ? kFaceY : kFaceX)) << (up ? 3 : 0);
+                    const int32_t inc = up ? 1 : -1;
+                    const Real at = up ? Real(0) : Real(1);
 #pragma unroll
-                            for (int a = 0; a < 3; ++a) {
-                                d[a] = n[a] * sc;
-                                if (!(T[a] < kNever)) continue;
-                                const Real dist = d[a] > Real(0) ? Real(1) - o[a] : o[a];
-                                T[a] = tau + __fdividef(dist, fabsf(d[a]));
+                    for (int a = 0; a < 3; ++a) {
+                        const bool p = a == best;
+                        o[a] = p ? at : clamp01(o[a] + dtt * d[a]);
+                        T[a] = p ? kNever : T[a];
+                        if (p) di[a] += inc;
+                    }
+                    if (!(fm & bit)) {
+                        bool changed = false;
+                        if (!membrane(best, up, ev, nv, changed)) {  // stays in its voxel, at the face
+                            nv = v;
+#pragma unroll
+                            for (int a = 0; a < 3; ++a)
+                                if (a == best) {
+                                    o[a] = Real(1) - at;
+                                    di[a] -= inc;
+                                }
+                        }
+                        if (changed) {
+                            const Real sn = __ldg(t.s + c);
+                            if (sn != sc) {
+                                sc = sn;
+#pragma unroll
+                                for (int a = 0; a < 3; ++a) {
+                                    d[a] = n[a] * sc;
+                                    if (!(T[a] < kNever)) continue;
+                                    const Real dist = d[a] > Real(0) ? Real(1) - o[a] : o[a];
+                                    T[a] = tau + mul_rcp(dist, fabsf(d[a]));
+                                }
                             }
                         }
+                    }
+                    v = nv;
+                    fm = __ldg(g.faces + v);
+                    if constexpr (IM != kInteractEC) {
+                        if (refused) break;
                     }
                 }
                 if (IM == kInteractEC || !refused) {
                     const Real rem = Real(1) - tau;
 #pragma unroll
                     for (int a = 0; a < 3; ++a) o[a] = clamp01(o[a] + rem * d[a]);
-                    if (t.any_relax) kahan_add(A, Ac, rem * rate);
+                    if (relax) kahan_add(A, Ac, rem * rate);
                 }
             }
             if constexpr (IM == kInteractEC) {
@@ -655,11 +702,12 @@ __device__ __forceinline__ void walk_block(const Geometry &g, const Tables<Real>
 #pragma unroll
                 for (int a = 0; a < 3; ++a) {
                     o[a] = o_s[a];
-                    wc[a] = wc_s[a];
                     di[a] = di_s[a];
                 }
                 v = v_s;
+                fm = fm_s;
                 c = c_s;
+                sc = sc_s;
                 A = A_s;
                 Ac = Ac_s;
                 if constexpr (HASH) {
@@ -672,7 +720,7 @@ __device__ __forceinline__ void walk_block(const Geometry &g, const Tables<Real>
                 }
                 if (IM == kInteractRS || ++att >= kMaxLeaps) {
                     // the walker stays for the step, in its label
-                    if (t.any_relax) {
+                    if (relax) {
                         if constexpr (kF64)
                             A = A + rate0;
                         else
@@ -683,63 +731,62 @@ __device__ __forceinline__ void walk_block(const Geometry &g, const Tables<Real>
                     break;
                 }
             }
-            }  // draws
-            if (HASH) {  // the verification kernel: checksum and, on request, invariants
-                const uint64_t x = (((uint64_t)k & 0xFFFFu) << 48) ^ ((uint64_t)(uint32_t)c << 32) ^
-                                   (uint64_t)(uint32_t)v;
-                h = mix64(h ^ x);
-                if (ctl.checked) {
-                    bool bad = false;
+        }  // draws
+        if constexpr (HASH) {  // the verification kernel: checksum and, on request, invariants
+            const uint64_t x =
+                (((uint64_t)k & 0xFFFFu) << 48) ^ ((uint64_t)(uint32_t)c << 32) ^ (uint64_t)(uint32_t)v;
+            h = mix64(h ^ x);
+            if (ctl.checked) {
+                int32_t at = 0;  // the flat index of the unwrapped coordinates
 #pragma unroll
-                    for (int a = 0; a < 3; ++a) bad = bad || wc[a] < 0 || wc[a] >= N[a];
-                    bad = bad || v != wc[0] + stride[1] * wc[1] + stride[2] * wc[2];
-                    if (!bad) bad = (int32_t)__ldg(g.labels + v) != c;  // indices checked first
+                for (int a = 0; a < 3; ++a) at += stride[a] * wrapped(st.i0[a][li] + di[a], N[a]);
+                bool bad = v != at;
+                // indices checked first
+                if (!bad) bad = (int32_t)__ldg(g.labels + v) != c || fm != __ldg(g.faces + v) || sc != __ldg(t.s + c);
 #pragma unroll
-                    for (int a = 0; a < 3; ++a) bad = bad || !(o[a] >= Real(0) && o[a] <= Real(1));
-                    if (bad) atomicOr(ctl.status, kErrInvariant);
-                }
+                for (int a = 0; a < 3; ++a) bad = bad || !(o[a] >= Real(0) && o[a] <= Real(1));
+                if (bad) atomicOr(ctl.status, kErrInvariant);
             }
-            // ---- phase (Eq. 7, right end point of each step)
-            if (fl & 1u) {
-                Real dx[3];
+        }
+        // ---- phase (Eq. 7, right end point of each step)
+        if (graded) {
+            Real dx[3];
 #pragma unroll
-                for (int a = 0; a < 3; ++a)
-                    dx[a] = mulr(lp, (Real)di[a] + (o[a] - o0[a]));
+            for (int a = 0; a < 3; ++a) dx[a] = mulr(lp, (Real)di[a] + (o[a] - o0[a]));
 #pragma unroll
-                for (int s = 0; s < NS; ++s) {
-                    if (s < ctl.n_shapes) {
-                        const Real wg = __ldg(t.wG + (int64_t)s * ctl.n_steps + (k - 1));
+            for (int s = 0; s < NS; ++s) {
+                if (s < ctl.n_shapes) {
+                    const Real wgs = NS == 1 ? wg : __ldg(t.wG + (int64_t)s * t.pitch + (k - 1));
 #pragma unroll
-                        for (int a = 0; a < 3; ++a) {
-                            if (kF64)
-                                ph[s][a] = ph[s][a] + dmul(wg, dx[a]);
-                            else
-                                kahan_add(ph[s][a], phc[s][a], wg * dx[a]);
-                        }
+                    for (int a = 0; a < 3; ++a) {
+                        if (kF64)
+                            ph[s][a] = ph[s][a] + dmul(wgs, dx[a]);
+                        else
+                            kahan_add(ph[s][a], phc[s][a], wgs * dx[a]);
                     }
                 }
             }
         }
         // ---- displacement moments at recording steps (block-uniform branch)
-        if (fl & 2u) {
-            double dx[3] = {0.0, 0.0, 0.0};
-            double al = 0.0;
-            if (active) {
+        if (k == next_rec) {
+            double dx[3];
 #pragma unroll
-                for (int a = 0; a < 3; ++a)
-                    dx[a] = g.voxel_um * ((double)di[a] + ((double)o[a] - (double)o0[a]));
-                al = kF64 ? exp(-(double)A) : exp(-((double)A - (double)Ac));
-            }
+            for (int a = 0; a < 3; ++a)
+                dx[a] = g.voxel_um * ((double)di[a] + ((double)o[a] - (double)o0[a]));
+            double al = 1.0;  // alpha = exp(-A); mostly A = 0 without relaxation
+            if (A != Real(0)) al = kF64 ? exp(-(double)A) : exp(-((double)A - (double)Ac));
+            if (!active) al = 0.0;
             warp_moments(al, dx, s_red[threadIdx.x >> 5]);
             __syncthreads();
             if (threadIdx.x < kMoments) {
                 double acc = 0.0;
 #pragma unroll
                 for (int ww = 0; ww < kWalkWarps; ++ww) acc += s_red[ww][threadIdx.x];
-                const int32_t r = __ldg(t.rec_of + (k - 1));
-                ctl.mom_partial[((int64_t)r * ctl.n_blocks + block) * kMoments + threadIdx.x] = acc;
+                ctl.mom_partial[((int64_t)rec * ctl.n_blocks + block) * kMoments + threadIdx.x] = acc;
             }
             __syncthreads();
+            ++rec;
+            next_rec = rec < ctl.n_rec ? __ldg(t.rec_step + rec) : INT32_MAX;
         }
     }
 
@@ -760,8 +807,8 @@ __device__ __forceinline__ void walk_block(const Geometry &g, const Tables<Real>
                     st.phase[((int64_t)s * 3 + a) * ctl.n_walkers + li] = ph[s][a];
                     if (!kF64) st.phase_c[((int64_t)s * 3 + a) * ctl.n_walkers + li] = phc[s][a];
                 }
-        if (HASH) st.hash[li] = h;
         if constexpr (HASH) {
+            st.hash[li] = h;
             if (st.counts) {
                 st.counts[li] = nev;
                 st.counts[ctl.n_walkers + li] = ncr;
@@ -775,24 +822,24 @@ __device__ __forceinline__ void walk_block(const Geometry &g, const Tables<Real>
 // the compiler's choice).  The plain form's one-shape kernel: its integer-ALU
 // arithmetic is made of long dependent chains, whose latency more warps hide,
 // and 5 blocks (at most 102 registers) measured 6 % faster than the
-// unconstrained 4.  The FP32 form's one-shape elastic-collision kernel: 9
-// blocks (56 registers, no spills; 36 warps per SM), 2.5 % faster than 7
-// blocks (72 registers) and 7.5 % faster than the compiler's own choice (80
-// registers, 6 blocks); 10 blocks spill.  The RS/ERL and absorbing-membrane
-// kernels would spill under such bounds, and kernels with more shapes keep
-// the registers their phases need.
+// unconstrained 4.  The FP32 form's one-shape elastic-collision kernel: 8
+// blocks (64 registers, 32 warps per SM), 21.8 ms for 1e6 walkers x 2000 steps
+// on 200x200x400 axons against 22.0 ms at 9 (56 registers, small spills) and
+// 22.5 ms at 7.  The RS/ERL and absorbing-membrane kernels would spill under
+// such bounds, and kernels with more shapes keep the registers their phases
+// need.
 template <typename Real, int NS, bool HASH, int IM, bool MT>
 constexpr int kWalkMinBlocks = (NS != 1) ? 0
                                : std::is_same<Real, double>::value ? 5
                                : (IM != kInteractEC || MT) ? 0
-                               : HASH ? 7 : 9;  // the verification kernel would spill at 9
+                               : HASH ? 7 : 8;  // the verification kernel would spill at 8
 
 // One run: block b of the grid advances walkers b*kWalkBlock ... of the run.
-template <typename Real, int NS, bool HASH, int IM, bool MT>
+template <typename Real, int NS, bool HASH, int IM, bool MT, int RELAX>
 __global__ void __launch_bounds__(kWalkBlock, kWalkMinBlocks<Real, NS, HASH, IM, MT>)
-walk_kernel(Geometry g, Tables<Real> t, WalkerState<Real> st, RunCtl ctl, int64_t k_begin, int64_t k_end)
+walk_kernel(Geometry g, Tables<Real> t, WalkerState<Real> st, RunCtl ctl, int64_t k_begin, int64_t k_end, int32_t rec)
 {
-    walk_block<Real, NS, HASH, IM, MT, true>(g, t, st, ctl, blockIdx.x, k_begin, k_end);
+    walk_block<Real, NS, HASH, IM, MT, RELAX, true>(g, t, st, ctl, blockIdx.x, k_begin, k_end, rec);
 }
 
 // Many runs in one launch (continuous batching): block i executes task i --
@@ -810,8 +857,8 @@ walk_batched_kernel(const ReqDesc<Real> *reqs, const BlockTask *tasks, int32_t n
         s_req = reqs[s_task.req];
     }
     __syncthreads();
-    walk_block<Real, NS, false, kInteractEC, false>(s_req.g, s_req.t, s_req.st, s_req.ctl, s_task.block,
-                                                    s_task.k0, s_task.k1);
+    walk_block<Real, NS, false, kInteractEC, false, 2>(s_req.g, s_req.t, s_req.st, s_req.ctl, s_task.block,
+                                                       s_task.k0, s_task.k1, s_task.rec);
 }
 
 template <typename Real>
@@ -856,25 +903,31 @@ int batched_blocks_per_sm(int ns_bucket)
 template <typename Real, int IM, bool MT>
 cudaError_t launch_walk(int n_shapes, bool hash, dim3 grid, cudaStream_t stream, const Geometry &g,
                         const Tables<Real> &t, const WalkerState<Real> &st, const RunCtl &ctl,
-                        int64_t k_begin, int64_t k_end)
+                        int64_t k_begin, int64_t k_end, int32_t rec)
 {
-#define RMS_LAUNCH(NSV)                                                                              \
-    do {                                                                                             \
-        if (hash)                                                                                    \
-            walk_kernel<Real, NSV, true, IM, MT><<<grid, kWalkBlock, 0, stream>>>(g, t, st, ctl,     \
-                                                                                 k_begin, k_end);    \
-        else                                                                                         \
-            walk_kernel<Real, NSV, false, IM, MT><<<grid, kWalkBlock, 0, stream>>>(g, t, st, ctl,    \
-                                                                                  k_begin, k_end);   \
+#define RMS_LAUNCH(NSV, HASHV, RELAXV)                                                                     \
+    walk_kernel<Real, NSV, HASHV, IM, MT, RELAXV><<<grid, kWalkBlock, 0, stream>>>(g, t, st, ctl, k_begin, \
+                                                                                  k_end, rec)
+#define RMS_LAUNCH_NS(HASHV, RELAXV)    \
+    do {                                \
+        if (n_shapes <= 1)              \
+            RMS_LAUNCH(1, HASHV, RELAXV); \
+        else if (n_shapes <= 2)         \
+            RMS_LAUNCH(2, HASHV, RELAXV); \
+        else if (n_shapes <= 4)         \
+            RMS_LAUNCH(4, HASHV, RELAXV); \
+        else                            \
+            RMS_LAUNCH(8, HASHV, RELAXV); \
     } while (0)
-    if (n_shapes <= 1)
-        RMS_LAUNCH(1);
-    else if (n_shapes <= 2)
-        RMS_LAUNCH(2);
-    else if (n_shapes <= 4)
-        RMS_LAUNCH(4);
+    if (hash)
+        RMS_LAUNCH_NS(true, 2);
+    else if constexpr (IM != kInteractEC || MT)
+        RMS_LAUNCH_NS(false, 2);
+    else if (t.any_relax)
+        RMS_LAUNCH_NS(false, 1);
     else
-        RMS_LAUNCH(8);
+        RMS_LAUNCH_NS(false, 0);
+#undef RMS_LAUNCH_NS
 #undef RMS_LAUNCH
     return cudaGetLastError();
 }

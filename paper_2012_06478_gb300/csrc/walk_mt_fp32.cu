@@ -7,11 +7,11 @@
 namespace rms {
 template cudaError_t launch_walk<float, kInteractEC, true>(int, bool, dim3, cudaStream_t, const Geometry &,
                                                     const Tables<float> &, const WalkerState<float> &,
-                                                    const RunCtl &, int64_t, int64_t);
+                                                    const RunCtl &, int64_t, int64_t, int32_t);
 template cudaError_t launch_walk<float, kInteractRS, true>(int, bool, dim3, cudaStream_t, const Geometry &,
                                                     const Tables<float> &, const WalkerState<float> &,
-                                                    const RunCtl &, int64_t, int64_t);
+                                                    const RunCtl &, int64_t, int64_t, int32_t);
 template cudaError_t launch_walk<float, kInteractERL, true>(int, bool, dim3, cudaStream_t, const Geometry &,
                                                     const Tables<float> &, const WalkerState<float> &,
-                                                    const RunCtl &, int64_t, int64_t);
+                                                    const RunCtl &, int64_t, int64_t, int32_t);
 }  // namespace rms

@@ -7,8 +7,8 @@
 namespace rms {
 template cudaError_t launch_walk<float, kInteractRS, false>(int, bool, dim3, cudaStream_t, const Geometry &,
                                                      const Tables<float> &, const WalkerState<float> &,
-                                                     const RunCtl &, int64_t, int64_t);
+                                                     const RunCtl &, int64_t, int64_t, int32_t);
 template cudaError_t launch_walk<float, kInteractERL, false>(int, bool, dim3, cudaStream_t, const Geometry &,
                                                       const Tables<float> &, const WalkerState<float> &,
-                                                      const RunCtl &, int64_t, int64_t);
+                                                      const RunCtl &, int64_t, int64_t, int32_t);
 }  // namespace rms
