@@ -259,38 +259,78 @@ __device__ __forceinline__ void neumaier(double &sum, double &comp, double x)
 
 // b of a unit waveform: b_s = dt sum_{j=1..N} F_{j-1}^2, F_j = F_{j-1} + dt G_j
 // (compensated sum); then q = sqrt(b / b_s), the amplitude giving b.  One
-// block per shape: the block stages the waveform through shared memory in
-// coalesced chunks and thread 0 takes the recurrence in step order -- the
-// CPU reference's operations in its order, so b_s is the same to the bit.
-// (Read straight from global memory, each step waited for its load: 34 ms
-// for N = 1e5, most of a sequence's set-up.)
+// block per shape, with the CPU reference's operations in its order, so b_s is
+// the same to the bit.
+//
+// What bounds it: three chains of N dependent additions (F, the sum, its
+// compensation), each one FP64 latency a step.  One thread doing all of a
+// step's operations -- two products and six or seven additions, each of which
+// holds GB300's narrow FP64 pipe as long as a whole warp's would -- was most of
+// a set-up: substrate, sequence of 6 shapes of 1e5 steps and a first run of 200
+// steps took 35.1 ms.  Here the chains run in three warps at once, each a chunk
+// behind the one before it, with only their own addition; the products F^2 and
+// dt G and the corrections, which no chain feeds back into, are done by all
+// threads between: 8.2 ms for the same calls.
 constexpr int kBvThreads = 256;
-constexpr int kBvChunk = 2048;
+constexpr int kBvChunk = 1024;
 
 __global__ void __launch_bounds__(kBvThreads) bvalue_kernel(int64_t N, int32_t S, double dt, const double *G,
                                                             int32_t n_b, const double *b, double *bs_out, double *q)
 {
     const int s = blockIdx.x;
     if (s >= S) return;  // block-uniform
-    __shared__ double sg[kBvChunk];
+    // a chunk's buffer holds dt G, then F before each step, then F^2, then the correction
+    __shared__ double buf[3][kBvChunk];
+    __shared__ double sums[2][kBvChunk + 1];  // the sum before each step of a chunk, and after its last
     const double *g = G + (int64_t)s * N;
-    double F = 0.0, sum = 0.0, comp = 0.0;  // thread 0's
-    for (int64_t base = 0; base < N; base += kBvChunk) {
-        const int n = (int)min((int64_t)kBvChunk, N - base);
-        for (int i = threadIdx.x; i < n; i += kBvThreads) sg[i] = g[base + i];
-        __syncthreads();
-        if (threadIdx.x == 0)
-            for (int i = 0; i < n; ++i) {
-                neumaier(sum, comp, F * F);
-                F = F + dt * sg[i];
+    const int chunks = (int)((N + kBvChunk - 1) / kBvChunk);
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    double chain = 0.0;  // lane 0 of warp 0: F; of warp 1: the sum; of warp 2: its compensation
+    for (int it = 0; it < chunks + 2; ++it) {
+        double *const b0 = buf[it % 3], *const b1 = buf[(it + 2) % 3], *const b2 = buf[(it + 1) % 3];
+        const auto length = [&](int c) {  // steps of chunk c (0: no such chunk)
+            return c < 0 || c >= chunks ? 0 : (int)min((int64_t)kBvChunk, N - (int64_t)c * kBvChunk);
+        };
+        const int n0 = length(it), n1 = length(it - 1), n2 = length(it - 2);
+        double *const t1 = sums[(it + 1) & 1];        // chunk it - 1
+        const double *const t2 = sums[it & 1];        // chunk it - 2
+        for (int i = threadIdx.x; i < kBvChunk; i += kBvThreads) {
+            if (i < n0) b0[i] = dt * g[(int64_t)it * kBvChunk + i];
+            if (i < n1) b1[i] = b1[i] * b1[i];
+            if (i < n2) {
+                const double x = b2[i], before = t2[i], t = t2[i + 1];
+                b2[i] = fabs(before) >= fabs(x) ? (before - t) + x : (x - t) + before;
             }
+        }
+        __syncthreads();
+        if (lane == 0 && warp < 3) {
+            if (warp == 0) {
+#pragma unroll 8
+                for (int i = 0; i < n0; ++i) {
+                    const double w = b0[i];
+                    b0[i] = chain;
+                    chain = chain + w;
+                }
+            } else if (warp == 1) {
+                t1[0] = chain;
+#pragma unroll 8
+                for (int i = 0; i < n1; ++i) {
+                    chain = chain + b1[i];
+                    t1[i + 1] = chain;
+                }
+            } else {
+#pragma unroll 8
+                for (int i = 0; i < n2; ++i) chain = chain + b2[i];
+            }
+        }
         __syncthreads();
     }
-    if (threadIdx.x == 0) {
-        const double bs = dt * (sum + comp);
-        bs_out[s] = bs;
-        for (int i = 0; i < n_b; ++i) q[s * n_b + i] = bs > 0.0 ? sqrt(b[i] / bs) : 0.0;
-    }
+    __shared__ double total[2];
+    if (lane == 0 && (warp == 1 || warp == 2)) total[warp - 1] = chain;
+    __syncthreads();
+    const double bs = dt * (total[0] + total[1]);
+    if (threadIdx.x == 0) bs_out[s] = bs;
+    for (int i = threadIdx.x; i < n_b; i += kBvThreads) q[s * n_b + i] = bs > 0.0 ? sqrt(b[i] / bs) : 0.0;
 }
 
 // ------------------------------------------------------------------ init (Sec. 2.2 item 1)
