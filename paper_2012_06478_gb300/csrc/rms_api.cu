@@ -418,72 +418,12 @@ __global__ void moments_reduce_kernel(const double *part, int32_t n_rec, int32_t
     out[idx] = s + c;
 }
 
-// Read-out (Eq. 7): for every (shape, direction, b) combination the sums of
-// alpha cos(phi) and -alpha sin(phi) over a chunk of walkers, phi = q (g . Phi_s),
-// alpha = exp(-A).  One thread per combination; the walkers of the chunk are
-// staged through shared memory in tiles.  The extra combination n_combo
+// The FP32 form's read-out: one thread per combination; the walkers of a chunk
+// are staged through shared memory in tiles.  The extra combination n_combo
 // carries the sum of alpha.
 constexpr int kRoBlock = 128;
 constexpr int kRoTile = 64;
 constexpr int64_t kRoChunk = 4096;
-
-template <typename Real>
-__global__ void __launch_bounds__(kRoBlock)
-readout_kernel(const Real *phase, const Real *phase_c, const Real *A, const Real *A_c, int64_t W, int32_t S,
-               const double *q, const double *dirs, int32_t n_dirs, int32_t n_b, int32_t n_combo,
-               double *part)
-{
-    __shared__ double sP[kRoTile][kMaxShapes * 3];
-    __shared__ double sAl[kRoTile];
-    const int combo = blockIdx.y * kRoBlock + threadIdx.x;  // grid: x = walker chunk, y = combination group
-    int s = 0;
-    double qq = 0.0, g0 = 0.0, g1 = 0.0, g2 = 0.0;
-    if (combo < n_combo) {
-        const int ib = combo % n_b;
-        const int gi = (combo / n_b) % n_dirs;
-        s = combo / (n_b * n_dirs);
-        qq = q[s * n_b + ib];
-        g0 = dirs[3 * gi];
-        g1 = dirs[3 * gi + 1];
-        g2 = dirs[3 * gi + 2];
-    }
-    const int64_t w0 = (int64_t)blockIdx.x * kRoChunk;
-    const int64_t w1 = min(W, w0 + kRoChunk);
-    double re = 0.0, im = 0.0;
-    for (int64_t base = w0; base < w1; base += kRoTile) {
-        const int nt = (int)min((int64_t)kRoTile, w1 - base);
-        for (int e = threadIdx.x; e < nt * (S * 3 + 1); e += kRoBlock) {
-            const int j = e % nt, k = e / nt;
-            const int64_t w = base + j;
-            if (k < S * 3) {
-                double p = (double)phase[(int64_t)k * W + w];
-                if (phase_c) p = p - (double)phase_c[(int64_t)k * W + w];
-                sP[j][k] = p;
-            } else {
-                double a = (double)A[w];
-                if (A_c) a = a - (double)A_c[w];
-                sAl[j] = exp(-a);
-            }
-        }
-        __syncthreads();
-        if (combo < n_combo) {
-            for (int j = 0; j < nt; ++j) {
-                const double phi = qq * (g0 * sP[j][3 * s] + g1 * sP[j][3 * s + 1] + g2 * sP[j][3 * s + 2]);
-                double sn, cs;
-                sincos(phi, &sn, &cs);
-                re += sAl[j] * cs;
-                im += -(sAl[j] * sn);
-            }
-        } else if (combo == n_combo) {
-            for (int j = 0; j < nt; ++j) re += sAl[j];
-        }
-        __syncthreads();
-    }
-    if (combo <= n_combo) {
-        part[((int64_t)blockIdx.x * (n_combo + 1) + combo) * 2 + 0] = re;
-        part[((int64_t)blockIdx.x * (n_combo + 1) + combo) * 2 + 1] = im;
-    }
-}
 
 // A float widened to double, exactly, on the integer ALU for normal values
 // and zeros (the FP64 pipe is GB300's scarce one); subnormals, infinities and
@@ -567,19 +507,6 @@ readout_f32_kernel(const float *phase, const float *phase_c, const float *A, con
         part[((int64_t)blockIdx.x * (n_combo + 1) + combo) * 2 + 0] = re;
         part[((int64_t)blockIdx.x * (n_combo + 1) + combo) * 2 + 1] = im;
     }
-}
-
-__global__ void readout_reduce_kernel(const double *part, int32_t n_chunks, int32_t n_combo, double *out)
-{
-    const int combo = blockIdx.x * blockDim.x + threadIdx.x;
-    if (combo > n_combo) return;
-    double rs = 0, rc = 0, is = 0, ic = 0;
-    for (int k = 0; k < n_chunks; ++k) {
-        neumaier(rs, rc, part[((int64_t)k * (n_combo + 1) + combo) * 2 + 0]);
-        neumaier(is, ic, part[((int64_t)k * (n_combo + 1) + combo) * 2 + 1]);
-    }
-    out[combo * 2 + 0] = rs + rc;
-    out[combo * 2 + 1] = is + ic;
 }
 
 // S = sum alpha e^{-i phi} / sum alpha from the unnormalised sums, which stay
@@ -1167,15 +1094,23 @@ static rms_status finalize_impl(rms_run_handle *r)
                                                                                 r->d_mom);
         RMS_CUDA(cudaGetLastError());
     }
-    const dim3 rgrid((unsigned)r->n_chunks, (unsigned)((r->n_combo + 1 + kRoBlock - 1) / kRoBlock));
-    if constexpr (std::is_same<Real, float>::value)
+    if constexpr (std::is_same<Real, float>::value) {
+        const dim3 rgrid((unsigned)r->n_chunks, (unsigned)((r->n_combo + 1 + kRoBlock - 1) / kRoBlock));
         readout_f32_kernel<<<rgrid, kRoBlock, 0, s>>>(st.phase, st.phase_c, st.A, st.A_c, r->W, q->S, q->d_q,
                                                       q->d_dirs, q->n_dirs, q->n_b, r->n_combo, r->d_ro_partial);
-    else
-        readout_kernel<Real><<<rgrid, kRoBlock, 0, s>>>(st.phase, st.phase_c, st.A, st.A_c, r->W, q->S, q->d_q,
-                                                        q->d_dirs, q->n_dirs, q->n_b, r->n_combo, r->d_ro_partial);
-    readout_reduce_kernel<<<(r->n_combo + 1 + 127) / 128, 128, 0, s>>>(r->d_ro_partial, r->n_chunks, r->n_combo,
-                                                                       r->d_S);
+        RMS_CUDA(cudaGetLastError());
+    } else {
+        ReadoutPlan p = readout_plan(r->W, q->S, q->n_dirs, q->n_b, INT32_MAX);
+        p.phase = st.phase;
+        p.sw = 1;
+        p.sk = r->W;
+        p.A = st.A;
+        p.q = q->d_q;
+        p.dirs = q->d_dirs;
+        p.part = r->d_ro_partial;
+        RMS_CUDA(launch_readout(p, s));
+    }
+    RMS_CUDA(launch_chunk_sums(r->d_ro_partial, r->n_chunks, r->n_combo, r->d_S, s));
     normalise_kernel<<<(r->n_combo + 1 + 127) / 128, 128, 0, s>>>(r->d_S, r->n_combo, normalised_S(r));
     RMS_CUDA(cudaGetLastError());
     return RMS_OK;
@@ -1200,13 +1135,20 @@ void rms::run_free(rms_run_handle *r, bool sync)
     if (r->ev_end) cudaEventDestroy(r->ev_end);
 }
 
+// Walker chunks of a form's read-out.
+static int64_t readout_chunks(const rms_sequence *q, int64_t W, int32_t precision)
+{
+    return precision == RMS_FP32 ? (W + kRoChunk - 1) / kRoChunk
+                                 : readout_plan(W, q->S, q->n_dirs, q->n_b, INT32_MAX).n_chunks;
+}
+
 size_t rms::run_state_bytes(const rms_sequence *q, int64_t W, int32_t precision, uint32_t flags)
 {
     WalkerState<double> s64{};
     WalkerState<float> s32{};
     const bool hash = (flags & kVerifyFlags) != 0;
     const int64_t nb = (W + kWalkBlockSize - 1) / kWalkBlockSize;
-    const int64_t nc = (W + kRoChunk - 1) / kRoChunk;
+    const int64_t nc = readout_chunks(q, W, precision);
     const int64_t ncombo = (int64_t)q->S * q->n_dirs * q->n_b;
     const bool cnt = (flags & RMS_COUNTS) != 0;
     const bool mort = (flags & RMS_MORTON) != 0;
@@ -1228,7 +1170,7 @@ rms_status rms::run_setup(rms_run_handle *r, bool with_cancel_and_events)
     const bool f32 = r->precision == RMS_FP32;
     r->n_blocks = (int32_t)((r->W + walk_block_size() - 1) / walk_block_size());
     r->n_combo = q->S * q->n_dirs * q->n_b;
-    r->n_chunks = (int32_t)((r->W + kRoChunk - 1) / kRoChunk);
+    r->n_chunks = (int32_t)readout_chunks(q, r->W, r->precision);
     const bool cnt = (r->flags & RMS_COUNTS) != 0;
     const bool mort = (r->flags & RMS_MORTON) != 0;
     const size_t bytes = f32 ? layout_state<float>(r->st32, nullptr, r->W, q->S, hash, true, cnt, mort)
