@@ -311,16 +311,6 @@ __global__ void __launch_bounds__(kBvThreads) bvalue_kernel(int64_t N, int32_t S
                     b0[i] = chain;
                     chain = chain + w;
                 }
-            } else if (warp == 1) {
-                t1[0] = chain;
-#pragma unroll 8
-                for (int i = 0; i < n1; ++i) {
-                    chain = chain + b1[i];
-                    t1[i + 1] = chain;
-                }
-            } else {
-#pragma unroll 8
-                for (int i = 0; i < n2; ++i) chain = chain + b2[i];
             }
         }
         __syncthreads();
@@ -416,97 +406,6 @@ __global__ void moments_reduce_kernel(const double *part, int32_t n_rec, int32_t
     double s = 0.0, c = 0.0;
     for (int b = 0; b < n_blocks; ++b) neumaier(s, c, part[((int64_t)r * n_blocks + b) * kMoments + m]);
     out[idx] = s + c;
-}
-
-// The FP32 form's read-out: one thread per combination; the walkers of a chunk
-// are staged through shared memory in tiles.  The extra combination n_combo
-// carries the sum of alpha.
-constexpr int kRoBlock = 128;
-constexpr int kRoTile = 64;
-constexpr int64_t kRoChunk = 4096;
-
-// A float widened to double, exactly, on the integer ALU for normal values
-// and zeros (the FP64 pipe is GB300's scarce one); subnormals, infinities and
-// NaNs take the hardware conversion, out of line so that it is not evaluated
-// speculatively beside the integer path.
-static __device__ __noinline__ double f2d_hw(float x) { return (double)x; }
-__device__ __forceinline__ double f2d(float x)
-{
-    const uint32_t b = __float_as_uint(x);
-    const uint32_t e = (b >> 23) & 0xFFu;
-    const uint64_t sign = (uint64_t)(b & 0x80000000u) << 32;
-    if (e == 0u) {
-        if ((b & 0x7FFFFFu) == 0u) return __longlong_as_double((long long)sign);  // +-0
-        return f2d_hw(x);
-    }
-    if (e == 0xFFu) return f2d_hw(x);
-    return __longlong_as_double((long long)(sign | ((uint64_t)(e + 896u) << 52) | ((uint64_t)(b & 0x7FFFFFu) << 29)));
-}
-
-// The FP32 form's read-out: the same sums over the same chunks in the same
-// order, with each term alpha e^{-i phi} evaluated in single precision --
-// the phase staged as the float nearest to its compensated value, phi =
-// q (g . Phi_s) and sincosf in FP32, alpha rounded to float -- and summed in
-// FP64 (the term widened exactly).  With P = q sum_i |g_i| |Phi_i| every term
-// is within about (6 P + 4) 2^-24 alpha of its FP64 value, so S is within
-// (6 P + 4) 2^-24 of the FP64 read-out of the same walkers (7.4e-6 at
-// P = 20 rad), far inside the form's 1e-3 bar on S; the per-walker terms do
-// not depend on the walkers' order or chunking.  b = 0 (q = 0) takes alpha
-// in FP64, so S(b = 0) = 1 exactly, and the sum of alpha stays FP64.
-__global__ void __launch_bounds__(kRoBlock)
-readout_f32_kernel(const float *phase, const float *phase_c, const float *A, const float *A_c, int64_t W, int32_t S,
-                   const double *q, const double *dirs, int32_t n_dirs, int32_t n_b, int32_t n_combo, double *part)
-{
-    __shared__ float sP[kRoTile][kMaxShapes * 3];
-    __shared__ float sAl[kRoTile];
-    __shared__ double sAlD[kRoTile];
-    const int combo = blockIdx.y * kRoBlock + threadIdx.x;
-    int s = 0;
-    float qq = 0.0f, g0 = 0.0f, g1 = 0.0f, g2 = 0.0f;
-    if (combo < n_combo) {
-        const int ib = combo % n_b;
-        const int gi = (combo / n_b) % n_dirs;
-        s = combo / (n_b * n_dirs);
-        qq = (float)q[s * n_b + ib];
-        g0 = (float)dirs[3 * gi];
-        g1 = (float)dirs[3 * gi + 1];
-        g2 = (float)dirs[3 * gi + 2];
-    }
-    const int64_t w0 = (int64_t)blockIdx.x * kRoChunk;
-    const int64_t w1 = min(W, w0 + kRoChunk);
-    double re = 0.0, im = 0.0;
-    for (int64_t base = w0; base < w1; base += kRoTile) {
-        const int nt = (int)min((int64_t)kRoTile, w1 - base);
-        for (int e = threadIdx.x; e < nt * (S * 3 + 1); e += kRoBlock) {
-            const int j = e % nt, k = e / nt;
-            const int64_t w = base + j;
-            if (k < S * 3) {
-                sP[j][k] = (float)((double)phase[(int64_t)k * W + w] - (double)phase_c[(int64_t)k * W + w]);
-            } else {
-                // kSaturatedF (saturated): exp underflows to 0
-                const double al = exp(-((double)A[w] - (double)A_c[w]));
-                sAlD[j] = al;
-                sAl[j] = (float)al;
-            }
-        }
-        __syncthreads();
-        if (combo < n_combo && qq != 0.0f) {
-            for (int j = 0; j < nt; ++j) {
-                const float gp = fmaf(g2, sP[j][3 * s + 2], fmaf(g1, sP[j][3 * s + 1], g0 * sP[j][3 * s]));
-                float sn, cs;
-                sincosf(qq * gp, &sn, &cs);
-                re += f2d(sAl[j] * cs);
-                im += f2d(-(sAl[j] * sn));
-            }
-        } else if (combo <= n_combo) {  // b = 0, and the sum of alpha
-            for (int j = 0; j < nt; ++j) re += sAlD[j];
-        }
-        __syncthreads();
-    }
-    if (combo <= n_combo) {
-        part[((int64_t)blockIdx.x * (n_combo + 1) + combo) * 2 + 0] = re;
-        part[((int64_t)blockIdx.x * (n_combo + 1) + combo) * 2 + 1] = im;
-    }
 }
 
 // S = sum alpha e^{-i phi} / sum alpha from the unnormalised sums, which stay
@@ -1094,22 +993,17 @@ static rms_status finalize_impl(rms_run_handle *r)
                                                                                 r->d_mom);
         RMS_CUDA(cudaGetLastError());
     }
-    if constexpr (std::is_same<Real, float>::value) {
-        const dim3 rgrid((unsigned)r->n_chunks, (unsigned)((r->n_combo + 1 + kRoBlock - 1) / kRoBlock));
-        readout_f32_kernel<<<rgrid, kRoBlock, 0, s>>>(st.phase, st.phase_c, st.A, st.A_c, r->W, q->S, q->d_q,
-                                                      q->d_dirs, q->n_dirs, q->n_b, r->n_combo, r->d_ro_partial);
-        RMS_CUDA(cudaGetLastError());
-    } else {
-        ReadoutPlan p = readout_plan(r->W, q->S, q->n_dirs, q->n_b, INT32_MAX);
-        p.phase = st.phase;
-        p.sw = 1;
-        p.sk = r->W;
-        p.A = st.A;
-        p.q = q->d_q;
-        p.dirs = q->d_dirs;
-        p.part = r->d_ro_partial;
-        RMS_CUDA(launch_readout(p, s));
-    }
+    ReadoutPlan<Real> p = readout_plan<Real>(r->W, q->S, q->n_dirs, q->n_b, INT32_MAX);
+    p.phase = st.phase;
+    p.phase_c = st.phase_c;
+    p.sw = 1;
+    p.sk = r->W;
+    p.A = st.A;
+    p.A_c = st.A_c;
+    p.q = q->d_q;
+    p.dirs = q->d_dirs;
+    p.part = r->d_ro_partial;
+    RMS_CUDA(launch_readout(p, s));
     RMS_CUDA(launch_chunk_sums(r->d_ro_partial, r->n_chunks, r->n_combo, r->d_S, s));
     normalise_kernel<<<(r->n_combo + 1 + 127) / 128, 128, 0, s>>>(r->d_S, r->n_combo, normalised_S(r));
     RMS_CUDA(cudaGetLastError());
@@ -1138,8 +1032,8 @@ void rms::run_free(rms_run_handle *r, bool sync)
 // Walker chunks of a form's read-out.
 static int64_t readout_chunks(const rms_sequence *q, int64_t W, int32_t precision)
 {
-    return precision == RMS_FP32 ? (W + kRoChunk - 1) / kRoChunk
-                                 : readout_plan(W, q->S, q->n_dirs, q->n_b, INT32_MAX).n_chunks;
+    return precision == RMS_FP32 ? readout_plan<float>(W, q->S, q->n_dirs, q->n_b, INT32_MAX).n_chunks
+                                 : readout_plan<double>(W, q->S, q->n_dirs, q->n_b, INT32_MAX).n_chunks;
 }
 
 size_t rms::run_state_bytes(const rms_sequence *q, int64_t W, int32_t precision, uint32_t flags)

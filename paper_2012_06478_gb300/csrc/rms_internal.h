@@ -45,18 +45,22 @@ extern template int batched_blocks_per_sm<float>(int);
 
 int walk_block_size();
 
-// The FP64 read-out (rms_readout.cu): phase component k of walker w at
-// phase[w sw + k sk] (one of the strides is 1); amplitudes q[shape][b], or
-// null: from b and b_s.  part: [n_chunks][n_combo + 1][2] sums, the last
-// column the sum of alpha.
+// The read-out (rms_readout.cu): phase component k of walker w at
+// phase[w sw + k sk] (one of the strides is 1); the compensations of the FP32
+// form likewise; amplitudes q[shape][b], or null: from b and b_s.  part:
+// [n_chunks][n_combo + 1][2] sums, the last column the sum of alpha.
+template <typename Real>
 struct ReadoutPlan {
-    const double *phase, *A, *q, *b, *b_s, *dirs;
+    const Real *phase, *phase_c, *A, *A_c;
+    const double *q, *b, *b_s, *dirs;
     int64_t sw, sk, W, per;
     double *part;
     int32_t S, n_dirs, n_b, n_combo, n_chunks, groups, cpb, nsub, threads, pitch;
 };
-ReadoutPlan readout_plan(int64_t W, int32_t S, int32_t n_dirs, int32_t n_b, int64_t max_chunks);
-cudaError_t launch_readout(const ReadoutPlan &p, cudaStream_t stream);
+template <typename Real>
+ReadoutPlan<Real> readout_plan(int64_t W, int32_t S, int32_t n_dirs, int32_t n_b, int64_t max_chunks);
+template <typename Real>
+cudaError_t launch_readout(const ReadoutPlan<Real> &p, cudaStream_t stream);
 cudaError_t launch_chunk_sums(const double *part, int32_t n_chunks, int32_t n_combo, double *out, cudaStream_t stream);
 cudaError_t launch_chunk_sums_normalised(const double *part, int32_t n_chunks, int32_t n_combo, double *S_re,
                                          double *S_im, double *alpha_sum, cudaStream_t stream);

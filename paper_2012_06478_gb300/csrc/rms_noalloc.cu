@@ -123,8 +123,8 @@ extern "C" rms_status rms_readout_noalloc(const double *phase, const double *A, 
     double *scratch = nullptr;
     rms_status st = scratch_ptr(&scratch);
     if (st != RMS_OK) return st;
-    rms::ReadoutPlan p =  // as many walker chunks as it would take, if they fit
-        rms::readout_plan(n_walkers, n_shapes, n_dirs, n_b, kScratchDoubles / per_chunk);
+    rms::ReadoutPlan<double> p =  // as many walker chunks as it would take, if they fit
+        rms::readout_plan<double>(n_walkers, n_shapes, n_dirs, n_b, kScratchDoubles / per_chunk);
     p.phase = phase;
     p.sw = 3 * (int64_t)n_shapes;
     p.sk = 1;

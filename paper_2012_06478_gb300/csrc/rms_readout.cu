@@ -1,7 +1,8 @@
-// rms_readout.cu -- the FP64 signal read-out (Eq. 7): for every (shape,
+// rms_readout.cu -- the signal read-out (Eq. 7): for every (shape,
 // direction, b) combination the sums over walkers of alpha cos(phi) and
-// -alpha sin(phi), phi = q (g . Phi_s), q = sqrt(b / b_s), alpha = exp(-A);
-// and the fixed-order sums over walker chunks of either form's read-out.
+// -alpha sin(phi), phi = q (g . Phi_s), q = sqrt(b / b_s), alpha = exp(-A), in
+// the plain form's 64-bit terms or the FP32 form's 32-bit ones; and the
+// fixed-order sums over walker chunks.
 #include <cuda_pipeline.h>
 #include <cuda_runtime.h>
 
@@ -19,46 +20,172 @@ __device__ const fix::Octant g_octant = fix::octant_table();
 constexpr int kTile = 64;         // walkers staged at a time: their exact sums fit 64 bits
 constexpr int kMaxThreads = 512;
 constexpr int kMaxPairs = 130;    // (shape, direction) pairs of one block's combinations, at most
-constexpr int kMinWalkers = 256;  // fewer: FP64 terms (their roundings are not averaged out)
+constexpr int kMinWalkers = 256;  // fewer: floating-point terms (their roundings are not averaged out)
 
-// A tile's terms in FP64: phases or alphas outside the integers' range.
-__device__ __noinline__ void plain_terms(const double *P, const double *al, int s, double q, double g0, double g1,
-                                         double g2, int first, int step, int n, double &re, double &im)
+// The forms' staged numbers: the plain form's terms are integers; the FP32
+// form's single precision (phi, sincosf and the product with alpha), with sums
+// that are exact but for the last places of a double.
+template <typename Real>
+struct Form;
+template <>
+struct Form<double> {
+    using Alpha = fix::Words;
+    using Phase = int64_t;
+    static constexpr int kBlocks = 2;  // resident blocks per SM
+    static constexpr size_t kTable = sizeof(fix::Angle) * fix::kAngles;
+};
+template <>
+struct Form<float> {
+    using Alpha = float;
+    using Phase = float;
+    static constexpr int kBlocks = 3;
+    static constexpr size_t kTable = sizeof(double) * 2 * kMaxThreads;  // the last sums' place
+};
+
+// alpha given in 58 bits of a power of two
+__device__ __forceinline__ void put(fix::Words &to, double, int64_t bits, int) { to = fix::words(bits); }
+// alpha over that power of two, below 1: x 2^(1022 - e)
+__device__ __forceinline__ void put(float &to, double al, int64_t, int e)
 {
-    const double *p = P + 3 * s * kTile;
+    to = (float)((double)(float)al * __longlong_as_double((long long)(2045 - e) << 52));
+}
+
+// The biased double exponent of the largest |x| of a warp's pairs of numbers.
+__device__ __forceinline__ int top_exponent(double a, double b)
+{
+    const unsigned u = (unsigned)(fix::double_word(a) >> 32) & 0x7FFFFFFFu;
+    const unsigned v = (unsigned)(fix::double_word(b) >> 32) & 0x7FFFFFFFu;
+    return (int)(__reduce_max_sync(0xffffffffu, max(u, v)) >> 20);
+}
+
+// Two single-precision numbers at a time (Blackwell's packed operations).
+struct F2 {
+    uint64_t v;
+};
+__device__ __forceinline__ F2 pair_of(float x, float y)
+{
+    F2 r;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(r.v) : "f"(x), "f"(y));
+    return r;
+}
+__device__ __forceinline__ float first(F2 a) { return __uint_as_float((uint32_t)a.v); }
+__device__ __forceinline__ float second(F2 a) { return __uint_as_float((uint32_t)(a.v >> 32)); }
+__device__ __forceinline__ F2 operator+(F2 a, F2 b)
+{
+    F2 r;
+    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r.v) : "l"(a.v), "l"(b.v));
+    return r;
+}
+__device__ __forceinline__ F2 operator-(F2 a, F2 b)
+{
+    F2 r;
+    asm("sub.rn.f32x2 %0, %1, %2;" : "=l"(r.v) : "l"(a.v), "l"(b.v));
+    return r;
+}
+
+// Sums of at most 64 pairs of numbers below 1: each is split at 2^-16 and 2^-33
+// by adding it to a number of fixed exponent, whose last place that is, so that
+// all sums but the last level's (below 2^-28) are exact.  Seven packed
+// additions, in place of two on the FP64 pipe.
+struct SplitSum {
+    static constexpr float kTop = 192.0f, kMid = 0x1.8p-10f;
+    F2 a = pair_of(kTop, kTop), b = pair_of(kMid, kMid), c = pair_of(0.0f, 0.0f);
+    __device__ __forceinline__ void add(F2 x)
+    {
+        const F2 ta = a + x;
+        x = x - (ta - a);
+        a = ta;
+        const F2 tb = b + x;
+        c = c + (x - (tb - b));
+        b = tb;
+    }
+    // one sum with 48 fraction bits
+    static __device__ __forceinline__ int64_t fixed(float a, float b, float c)
+    {
+        return ((int64_t)(__float_as_int(a) - __float_as_int(kTop)) << 32) +
+               ((int64_t)(__float_as_int(b) - __float_as_int(kMid)) << 15) + __float2int_rn(c * 0x1p48f);
+    }
+};
+
+// g.Phi of walker j's staged phases (the FP32 form's with their compensations).
+__device__ __forceinline__ double dot(const double *v, int, int j, const double *g)
+{
+    return fma(g[2], v[2 * kTile + j], fma(g[1], v[kTile + j], g[0] * v[j]));
+}
+__device__ __forceinline__ float dot(const float *v, int K, int j, const double *g)
+{
+    const float *c = v + K * kTile;
+    return fmaf((float)g[2], v[2 * kTile + j] - c[2 * kTile + j],
+                fmaf((float)g[1], v[kTile + j] - c[kTile + j], (float)g[0] * (v[j] - c[j])));
+}
+
+// A tile's sums in floating point: phases or alphas outside the integers' range.
+__device__ __noinline__ double2 plain_sums(const double *v, int, const double *al, double q, const double *g, int first,
+                                           int step, int n)
+{
+    double re = 0.0, im = 0.0;
     for (int j = first; j < n; j += step) {
-        const double phi = q * (g0 * p[j] + g1 * p[kTile + j] + g2 * p[2 * kTile + j]);
+        const double phi = q * (g[0] * v[j] + g[1] * v[kTile + j] + g[2] * v[2 * kTile + j]);
         double sn, cs;
         sincos(phi, &sn, &cs);
         re += al[j] * cs;
         im += -(al[j] * sn);
     }
+    return make_double2(re, im);
+}
+__device__ __noinline__ double2 plain_sums(const float *v, int K, const double *al, double q, const double *g,
+                                           int first, int step, int n)
+{
+    double re = 0.0, im = 0.0;
+    for (int j = first; j < n; j += step) {
+        const float phi = (float)q * dot(v, K, j, g);
+        float sn, cs;
+        sincosf(phi, &sn, &cs);
+        re += (double)((float)al[j] * cs);
+        im += (double)-((float)al[j] * sn);
+    }
+    return make_double2(re, im);
+}
+
+template <typename Real>
+constexpr size_t smem_bytes(int S, int pitch)
+{
+    using F = Form<Real>;
+    const int rows = (sizeof(Real) == 8 ? 1 : 2) * (3 * S + 1);
+    return F::kTable + sizeof(double) * kTile + sizeof(Real) * 2 * rows * kTile + sizeof(typename F::Alpha) * kTile +
+           sizeof(typename F::Phase) * kTile * pitch + sizeof(int) * pitch;
 }
 
 // Grid: x a group of p.cpb combinations, y a chunk of p.per walkers.  A thread
 // has one combination and every p.nsub-th walker of the chunk.
 //
-// What bounds it: issue (about 70 instructions a term, a third of them 32-bit
-// products of 64 bits).  1e6 walkers x 330 combinations: RO_AFTER ms, against
-// RO_BEFORE ms with sincos and sums on the FP64 pipe.  Tiles of 64 walkers go
-// through shared memory twice -- the walkers' phases, copied asynchronously
-// while the tile before is summed, and g.Phi of every pair in fixed point,
-// shared by the pair's b-values -- beside the 64 KiB table, which two blocks an
-// SM amortise over all their walkers.
-__global__ void __launch_bounds__(kMaxThreads, 2) readout_fixed_kernel(ReadoutPlan p)
+// What bounds it: issue, and the pipe of the 32-bit products (plain form, 1e6
+// walkers x 330 combinations: 57 % and 72 % used).  2.69 ms there, against 25.6
+// with sincos and sums on the FP64 pipe; the FP32 form, whose sums on the FP64
+// pipe took 31.9 ms for 1e7 walkers x 512 combinations, 11.7 ms.
+// Tiles of 64 walkers go through shared memory twice -- the walkers' phases,
+// copied asynchronously while the tile before is summed, and g.Phi of every
+// pair (the plain form's in fixed point), shared by the pair's b-values; the
+// table of the plain form is amortised over all of a block's walkers.
+template <typename Real>
+__global__ void __launch_bounds__(kMaxThreads, Form<Real>::kBlocks) readout_fixed_kernel(ReadoutPlan<Real> p)
 {
+    using F = Form<Real>;
+    constexpr bool kF64 = sizeof(Real) == 8;
     extern __shared__ __align__(16) char smem[];
-    fix::Angle *const table = (fix::Angle *)smem;
-    const int K = 3 * p.S, row = K + 1;  // staged numbers of a walker: its phases and A
-    double *const raw = (double *)(table + fix::kAngles);  // [2][row][kTile]
-    double *const alD = raw + 2 * row * kTile;              // alpha of the tile
-    fix::Words *const alF = (fix::Words *)(alD + kTile);   // in 58 bits of the largest
-    int64_t *const X = (int64_t *)(alF + kTile);            // [kTile][pitch]
-    int *const em = (int *)(X + kTile * p.pitch);           // per pair: the largest |g.Phi|'s exponent
+    auto *const table = (fix::Angle *)smem;  // plain form
+    // staged numbers of a walker: its phases and A (FP32 form: phases, compensations, A and A's)
+    const int K = 3 * p.S, KA = kF64 ? K : 2 * K, rows = kF64 ? K + 1 : 2 * K + 2;
+    double *const alD = (double *)(smem + F::kTable);                 // alpha of the tile
+    Real *const raw = (Real *)(alD + kTile);                          // [2][rows][kTile]
+    auto *const alF = (typename F::Alpha *)(raw + 2 * rows * kTile);  // over a power of two above the largest
+    auto *const X = (typename F::Phase *)(alF + kTile);               // [kTile][pitch]
+    int *const em = (int *)(X + kTile * p.pitch);                     // per pair: the largest |g.Phi|'s exponent
     __shared__ double s_asum;
-    __shared__ int s_ea;  // exponent of the tile's largest alpha; 0: FP64 terms
+    __shared__ int s_ea;  // exponent of the tile's largest alpha; 0: floating-point terms
 
-    for (int k = threadIdx.x; k < fix::kAngles; k += blockDim.x) table[k] = fix::angle_of(g_octant, k);
+    if constexpr (kF64)
+        for (int k = threadIdx.x; k < fix::kAngles; k += blockDim.x) table[k] = fix::angle_of(g_octant, k);
 
     const int64_t c0 = (int64_t)blockIdx.x * p.cpb;
     const int n_here = (int)min((int64_t)p.cpb, p.n_combo - c0);
@@ -66,59 +193,67 @@ __global__ void __launch_bounds__(kMaxThreads, 2) readout_fixed_kernel(ReadoutPl
     const int sub = threadIdx.x / p.cpb, mine = threadIdx.x - sub * p.cpb;
     const bool active = sub < p.nsub && mine < n_here;
     int s = 0, pair = 0;
-    double q = 0.0, g0 = 0.0, g1 = 0.0, g2 = 0.0;
+    double q = 0.0;
+    const double *g = p.dirs;
     if (active) {
         const int combo = (int)(c0 + mine), ib = combo % p.n_b;
         pair = combo / p.n_b;
         s = pair / p.n_dirs;
         q = p.q ? p.q[s * p.n_b + ib] : (p.b_s[s] > 0.0 ? sqrt(p.b[ib] / p.b_s[s]) : 0.0);
-        const double *g = p.dirs + 3 * (pair - s * p.n_dirs);
-        g0 = g[0];
-        g1 = g[1];
-        g2 = g[2];
+        g = p.dirs + 3 * (pair - s * p.n_dirs);
         pair -= pair0;
     }
     const int64_t Q = fix::turns_of(q);
 
     const int64_t w0 = (int64_t)blockIdx.y * p.per, w1 = min(p.W, w0 + p.per);
-    const auto stage = [&](int64_t base, double *to) {  // asynchronous copy of a tile's walkers
+    const auto stage = [&](int64_t base, Real *to) {  // asynchronous copy of a tile's walkers
         const int nt = (int)min((int64_t)kTile, w1 - base);
-        for (int e = threadIdx.x; e < row * kTile; e += blockDim.x) {
+        for (int e = threadIdx.x; e < rows * kTile; e += blockDim.x) {
             // neighbouring threads take neighbouring numbers of memory
-            const int j = p.sw == 1 ? e % kTile : e / row, k = p.sw == 1 ? e / kTile : e % row;
+            const int j = p.sw == 1 ? e % kTile : e / rows, k = p.sw == 1 ? e / kTile : e % rows;
             if (j >= nt) continue;
-            const double *from = k < K ? p.phase + (base + j) * p.sw + k * p.sk : p.A + base + j;
-            __pipeline_memcpy_async(to + k * kTile + j, from, sizeof(double));
+            const Real *from;
+            if (k < K)
+                from = p.phase + (base + j) * p.sw + k * p.sk;
+            else if (k < KA)
+                from = p.phase_c + (base + j) * p.sw + (k - K) * p.sk;
+            else
+                from = (k == KA ? p.A : p.A_c) + base + j;
+            __pipeline_memcpy_async(to + k * kTile + j, from, sizeof(Real));
         }
         __pipeline_commit();
     };
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, n_warps = (blockDim.x + 31) >> 5;
     double re = 0.0, im = 0.0, asum = 0.0;
+    // FP32 form: the sums of the tiles so far that had their alphas' exponent, 48 fraction bits
+    [[maybe_unused]] int64_t re48 = 0, im48 = 0;
+    [[maybe_unused]] int ea48 = 0, tiles48 = 0;
+    [[maybe_unused]] const auto flush = [&] {
+        const double scale = __longlong_as_double((long long)(ea48 - 47) << 52);  // 2^(ea48 - 1022 - 48)
+        re += (double)re48 * scale;
+        im -= (double)im48 * scale;
+        re48 = im48 = tiles48 = 0;
+    };
     stage(w0, raw);
     int at = 0;
     for (int64_t base = w0; base < w1; base += kTile, at ^= 1) {
         const int nt = (int)min((int64_t)kTile, w1 - base);
-        double *const P = raw + at * row * kTile;
+        Real *const P = raw + at * rows * kTile;
         __pipeline_wait_prior(0);
         __syncthreads();  // the tile has come, and the sums of the one before are done
-        if (base + kTile < w1) stage(base + kTile, raw + (at ^ 1) * row * kTile);
+        if (base + kTile < w1) stage(base + kTile, raw + (at ^ 1) * rows * kTile);
         // a warp each: alpha, and g.Phi of one pair at a time
         for (int t = warp; t <= n_pairs; t += n_warps) {
-            double x[2];
             if (t == n_pairs) {
-                for (int h = 0; h < 2; ++h) x[h] = lane + 32 * h < nt ? exp(-P[K * kTile + lane + 32 * h]) : 0.0;
-            } else {
-                const int ps = (pair0 + t) / p.n_dirs;
-                const double *g = p.dirs + 3 * (pair0 + t - ps * p.n_dirs), *v = P + 3 * ps * kTile;
+                double x[2];
                 for (int h = 0; h < 2; ++h) {
                     const int j = lane + 32 * h;
-                    x[h] = j < nt ? fma(g[2], v[2 * kTile + j], fma(g[1], v[kTile + j], g[0] * v[j])) : 0.0;
+                    double a = j < nt ? (double)P[KA * kTile + j] : 0.0;
+                    if (!kF64 && j < nt) a = a - (double)P[(KA + 1) * kTile + j];
+                    // kSaturatedF (saturated, FP32 form): exp underflows to 0
+                    x[h] = j < nt ? exp(-a) : 0.0;
                 }
-            }
-            const unsigned top = max((unsigned)(fix::double_word(x[0]) >> 32) & 0x7FFFFFFFu,
-                                     (unsigned)(fix::double_word(x[1]) >> 32) & 0x7FFFFFFFu);
-            const int e = (int)(__reduce_max_sync(0xffffffffu, top) >> 20);
-            if (t == n_pairs) {
+                const int e = top_exponent(x[0], x[1]);
                 // within 2^+-900: the scaled sums stay in range
                 const bool fixed = e > 123 && e < 1923 && p.W >= kMinWalkers;
                 double sum;
@@ -126,7 +261,7 @@ __global__ void __launch_bounds__(kMaxThreads, 2) readout_fixed_kernel(ReadoutPl
                     uint64_t n = 0;  // 64 numbers below 2^58: exact
                     for (int h = 0; h < 2; ++h) {
                         const int64_t f = fix::scaled(x[h], e, 58);
-                        alF[lane + 32 * h] = fix::words(f);
+                        put(alF[lane + 32 * h], x[h], f, e);
                         n += (uint64_t)f;
                     }
                     for (int o = 16; o > 0; o >>= 1) n += __shfl_xor_sync(0xffffffffu, n, o);
@@ -142,32 +277,80 @@ __global__ void __launch_bounds__(kMaxThreads, 2) readout_fixed_kernel(ReadoutPl
                     s_ea = fixed ? e : 0;
                 }
             } else {
-                for (int h = 0; h < 2; ++h) X[(lane + 32 * h) * p.pitch + t] = fix::scaled(x[h], e, 62);
-                if (lane == 0) em[t] = e;
+                const int ps = (pair0 + t) / p.n_dirs;
+                const double *gt = p.dirs + 3 * (pair0 + t - ps * p.n_dirs);
+                Real x[2];
+                for (int h = 0; h < 2; ++h)
+                    x[h] = lane + 32 * h < nt ? dot(P + 3 * ps * kTile, K, lane + 32 * h, gt) : Real(0);
+                if constexpr (kF64) {
+                    const int e = top_exponent(x[0], x[1]);
+                    for (int h = 0; h < 2; ++h) X[(lane + 32 * h) * p.pitch + t] = fix::scaled(x[h], e, 62);
+                    if (lane == 0) em[t] = e;
+                } else {
+                    for (int h = 0; h < 2; ++h) X[(lane + 32 * h) * p.pitch + t] = x[h];
+                }
             }
         }
         __syncthreads();
         const int ea = s_ea;
         if (threadIdx.x == 0) asum += s_asum;
         if (active) {
-            const fix::Scale sc = fix::scale_of(q, Q, em[pair]);
-            if (q == 0.0 && em[pair] < 0x7FF) {  // b = 0: alpha's own sum, so that S = 1 exactly
+            bool alphas;  // b = 0: alpha's own sum, so that S = 1 exactly
+            bool fixed = ea != 0;
+            fix::Scale sc;
+            if constexpr (kF64) {
+                sc = fix::scale_of(q, Q, em[pair]);
+                alphas = q == 0.0 && em[pair] < 0x7FF;
+                fixed = fixed && sc.ok;
+            } else {
+                alphas = (float)q == 0.0f;
+            }
+            if (alphas) {
                 if (sub == 0) {
                     re += s_asum;
-                    im -= 0.0 * s_asum;
+                    if constexpr (kF64) im -= 0.0 * s_asum;
                 }
-            } else if (sc.ok && ea) {
-                int64_t c = 0, sn = 0;
-                for (int j = sub; j < nt; j += p.nsub)
-                    fix::add_term(X[j * p.pitch + pair], sc, alF[j], table, c, sn);
-                const double scale = __longlong_as_double((long long)(ea - 55) << 52);  // 2^(ea - 1022 - 56)
-                re += (double)c * scale;
-                im -= (double)sn * scale;
+            } else if (fixed) {
+                if constexpr (kF64) {
+                    int64_t c = 0, sn = 0;
+#pragma unroll 4
+                    for (int j = sub; j < nt; j += p.nsub)
+                        fix::add_term(X[j * p.pitch + pair], sc, alF[j], table, c, sn);
+                    const double scale = __longlong_as_double((long long)(ea - 55) << 52);  // 2^(ea - 1022 - 56)
+                    re += (double)c * scale;
+                    im -= (double)sn * scale;
+                } else {
+                    SplitSum sum;
+                    const float qq = (float)q;
+#pragma unroll 2
+                    for (int j = sub; j < nt; j += p.nsub) {
+                        float sn, cs;
+                        sincosf(qq * X[j * p.pitch + pair], &sn, &cs);
+                        sum.add(pair_of(alF[j] * cs, alF[j] * sn));
+                    }
+                    if (ea != ea48 || tiles48 == 256) {
+                        if (tiles48) flush();
+                        ea48 = ea;
+                    }
+                    // a phase that is not finite makes the sum NaN, not an integer
+                    if (isnan(first(sum.c)) || isnan(second(sum.c))) {
+                        re += (double)first(sum.c);
+                        im += (double)second(sum.c);
+                    } else {
+                        re48 += SplitSum::fixed(first(sum.a), first(sum.b), first(sum.c));
+                        im48 += SplitSum::fixed(second(sum.a), second(sum.b), second(sum.c));
+                        ++tiles48;
+                    }
+                }
             } else {
-                plain_terms(P, alD, s, q, g0, g1, g2, sub, p.nsub, nt, re, im);
+                const double2 r = plain_sums(P + 3 * s * kTile, K, alD, q, g, sub, p.nsub, nt);
+                re += r.x;
+                im += r.y;
             }
         }
     }
+    if constexpr (!kF64)
+        if (tiles48) flush();
     // over a combination's threads, in order
     __syncthreads();
     double *const red = (double *)smem;  // [nsub][cpb][2]: at most 8 KiB, where the table was
@@ -203,10 +386,10 @@ __device__ __forceinline__ void neumaier(double &sum, double &comp, double x)
 
 // Sums over walker chunks in a fixed order.  A block has 32 combinations; its
 // eight warps take every eighth chunk each (one thread over all chunks took
-// SUM_BEFORE us for 2442 chunks x 513 combinations, a chain of dependent FP64
-// additions; eight at once, SUM_AFTER us).  NORM: the last column, the sum of
-// alpha, divides the others (split real and imaginary parts, alpha_sum
-// optional); otherwise all n_combo + 1 sums as they are.
+// 233 us for 2442 chunks x 513 combinations, a chain of dependent FP64
+// additions; eight at once, and fewer chunks, 48 us).  NORM: the last column,
+// the sum of alpha, divides the others (split real and imaginary parts,
+// alpha_sum optional); otherwise all n_combo + 1 sums as they are.
 constexpr int kSumWarps = 8;
 
 template <bool NORM>
@@ -249,11 +432,12 @@ chunk_sums_kernel(const double *part, int32_t n_chunks, int32_t n_combo, double 
 
 // How the read-out splits: combinations a block (one group when they fit its
 // threads, at most kMaxPairs pairs), threads a combination, and walkers a
-// block -- a whole wave of two blocks an SM for few groups, four waves (whose
-// last is less empty) for many, whole tiles, at most max_chunks chunks.
-ReadoutPlan readout_plan(int64_t W, int32_t S, int32_t n_dirs, int32_t n_b, int64_t max_chunks)
+// block -- a whole wave of the blocks that are resident for few groups, four
+// waves (whose last is less empty) for many, whole tiles, at most max_chunks.
+template <typename Real>
+ReadoutPlan<Real> readout_plan(int64_t W, int32_t S, int32_t n_dirs, int32_t n_b, int64_t max_chunks)
 {
-    ReadoutPlan p{};
+    ReadoutPlan<Real> p{};
     p.W = W;
     p.S = S;
     p.n_dirs = n_dirs;
@@ -267,7 +451,7 @@ ReadoutPlan readout_plan(int64_t W, int32_t S, int32_t n_dirs, int32_t n_b, int6
     p.threads = (p.cpb * p.nsub + 31) / 32 * 32;
     p.groups = (int32_t)groups;
     p.pitch = (int32_t)std::min<int64_t>((int64_t)S * n_dirs, (p.cpb - 1) / n_b + 2) | 1;  // odd: no bank conflicts
-    constexpr int64_t kWave = 2 * 152;
+    constexpr int64_t kWave = Form<Real>::kBlocks * 152;
     int64_t chunks = std::max<int64_t>(1, (groups <= 8 ? kWave : 4 * kWave) / groups);
     chunks = std::min(std::min(chunks, (W + kTile - 1) / kTile), max_chunks);
     p.per = ((W + chunks - 1) / chunks + kTile - 1) / kTile * kTile;
@@ -275,25 +459,25 @@ ReadoutPlan readout_plan(int64_t W, int32_t S, int32_t n_dirs, int32_t n_b, int6
     return p;
 }
 
-static constexpr size_t smem_bytes(int S, int pitch)
-{
-    return sizeof(fix::Angle) * fix::kAngles + sizeof(double) * 2 * (3 * S + 1) * kTile + 2 * sizeof(double) * kTile +
-           sizeof(int64_t) * kTile * pitch + sizeof(int) * pitch;
-}
-
-cudaError_t launch_readout(const ReadoutPlan &p, cudaStream_t stream)
+template <typename Real>
+cudaError_t launch_readout(const ReadoutPlan<Real> &p, cudaStream_t stream)
 {
     // the largest any plan needs, so that host threads do not set different limits;
     // per context, and cheap: asked for at every launch
-    constexpr size_t kMost = smem_bytes(kMaxShapes, kMaxPairs | 1);
+    constexpr size_t kMost = smem_bytes<Real>(kMaxShapes, kMaxPairs | 1);
     static_assert(kMost <= 227 * 1024, "shared memory of a block");
     const cudaError_t e =
-        cudaFuncSetAttribute(readout_fixed_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kMost);
+        cudaFuncSetAttribute(readout_fixed_kernel<Real>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kMost);
     if (e != cudaSuccess) return e;
-    readout_fixed_kernel<<<dim3((unsigned)p.groups, (unsigned)p.n_chunks), p.threads, smem_bytes(p.S, p.pitch),
-                           stream>>>(p);
+    readout_fixed_kernel<Real><<<dim3((unsigned)p.groups, (unsigned)p.n_chunks), p.threads,
+                                 smem_bytes<Real>(p.S, p.pitch), stream>>>(p);
     return cudaGetLastError();
 }
+
+template ReadoutPlan<double> readout_plan<double>(int64_t, int32_t, int32_t, int32_t, int64_t);
+template ReadoutPlan<float> readout_plan<float>(int64_t, int32_t, int32_t, int32_t, int64_t);
+template cudaError_t launch_readout<double>(const ReadoutPlan<double> &, cudaStream_t);
+template cudaError_t launch_readout<float>(const ReadoutPlan<float> &, cudaStream_t);
 
 cudaError_t launch_chunk_sums(const double *part, int32_t n_chunks, int32_t n_combo, double *out, cudaStream_t stream)
 {

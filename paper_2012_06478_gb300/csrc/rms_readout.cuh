@@ -154,9 +154,9 @@ __host__ __device__ __forceinline__ void add_term(int64_t X, const Scale &q, Wor
     const int64_t s = R + mul_ss(r3, -(1 << 17));  // sin r + 2^31, so that the low word is signed
     const int32_t sh = hi32(s), sl = (int32_t)(lo32(s) ^ 0x80000000u);
     // cos(a + r) = C + (C (cos r - 1) - S sin r), sin(a + r) = S + (S (cos r - 1) + C sin r)
-    const int64_t zc = mul_ss(a.c.hi, m) + ((mul_ss(a.s.hi, -sl) + mul_ss(a.s.lo, -sh)) >> 20);
+    const int64_t zc = mul_ss(a.c.hi, m) + (-(mul_ss(a.s.hi, sl) + mul_ss(a.s.lo, sh)) >> 20);
     const int64_t zs = mul_ss(a.s.hi, m) + ((mul_ss(a.c.hi, sl) + mul_ss(a.c.lo, sh)) >> 20);
-    const int64_t yc = mul_ss(a.s.hi, -sh) + (zc >> 12);
+    const int64_t yc = (zc >> 12) - mul_ss(a.s.hi, sh);
     const int64_t ys = mul_ss(a.c.hi, sh) + (zs >> 12);
     const int64_t cs = (yc >> 8) + a.c.lo + (int64_t)((uint64_t)(uint32_t)a.c.hi << 32);
     const int64_t sn = (ys >> 8) + a.s.lo + (int64_t)((uint64_t)(uint32_t)a.s.hi << 32);
