@@ -375,19 +375,26 @@ __global__ void init_kernel(Geometry g, const int32_t *ok_list, int64_t n_ok, co
 // Moments, first level: the per-block partials of recording step r, blocks
 // c*kMomChunk ..., staged through shared memory with coalesced loads (the
 // partials of one recording step are contiguous), each of the 22 sums taken
-// in block order with compensation.  Block index = r * n_mchunks + c.
+// in block order with compensation.  A block's partial is the sum of `sub` of
+// them, in order (1, or the four warps' of a block).  Block index = r *
+// n_mchunks + c.
 constexpr int kMomChunk = 256;
 
-__global__ void __launch_bounds__(256) moments_chunk_kernel(const double *part, int32_t n_blocks, int32_t n_mchunks,
-                                                            double *out)
+__global__ void __launch_bounds__(256) moments_chunk_kernel(const double *part, int32_t n_blocks, int32_t sub,
+                                                            int32_t n_mchunks, double *out)
 {
     __shared__ double tile[kMomChunk * kMoments];
     const int64_t r = blockIdx.x / n_mchunks;
     const int32_t c = blockIdx.x % n_mchunks;
     const int32_t b0 = c * kMomChunk;
     const int32_t nb = min(kMomChunk, n_blocks - b0);
-    const double *src = part + (r * n_blocks + b0) * kMoments;
-    for (int e = threadIdx.x; e < nb * kMoments; e += blockDim.x) tile[e] = src[e];
+    const double *src = part + (r * n_blocks + b0) * sub * kMoments;
+    for (int e = threadIdx.x; e < nb * kMoments; e += blockDim.x) {
+        const double *p = src + (int64_t)(e / kMoments) * sub * kMoments + e % kMoments;
+        double acc = p[0];
+        for (int k = 1; k < sub; ++k) acc += p[k * kMoments];
+        tile[e] = acc;
+    }
     __syncthreads();
     if (threadIdx.x < kMoments) {
         double sum = 0.0, comp = 0.0;
@@ -953,6 +960,11 @@ static rms_status walk_impl(rms_run_handle *r, int64_t k0, int64_t k1)
     const dim3 grid((unsigned)r->n_blocks);
     const int S = r->seq->S;
     const int32_t rec = first_rec(r->seq, k0);
+    if constexpr (std::is_same<Real, double>::value)
+        if (r->quad) {
+            RMS_CUDA(launch_walk_quad(S, r->stream, d.g, d.t, d.st, d.ctl, k0, k1, rec));
+            return RMS_OK;
+        }
 #define RMS_WALK(IM, MT) \
     RMS_CUDA((launch_walk<Real, IM, MT>(S, hash, grid, r->stream, d.g, d.t, d.st, d.ctl, k0, k1, rec)))
     const bool mt = d.t.Tmt != nullptr;
@@ -976,6 +988,17 @@ rms_status rms::run_walk(rms_run_handle *r, int64_t k0, int64_t k1)
     return r->precision == RMS_FP32 ? walk_impl<float>(r, k0, k1) : walk_impl<double>(r, k0, k1);
 }
 
+// Plain-form runs of at most this many walkers take four lanes to a walker: two
+// waves of its blocks (five of 32 walkers an SM).  600 steps of 500, 1e4, 2e4 and
+// 4e4 walkers in axons: 1.95, 2.39, 3.12 and 5.14 ms against 4.41, 4.52, 5.31 and
+// 6.46; with relaxation and unequal D 2.09, 2.62, 3.47 and 5.71 against 4.45,
+// 4.59, 5.42 and 6.54.  In a third wave the one-thread kernel's fewer
+// instructions win (5e4: 6.98 against 6.75).
+constexpr int64_t kQuadMaxWalkers = 2 * 5 * 152 * 32;
+
+// Moment partials of a block of the walk.
+static int32_t mom_sub(const rms_run_handle *r) { return r->quad ? kWalkBlockSize / 32 : 1; }
+
 static int32_t mom_chunks(int32_t n_blocks) { return (n_blocks + kMomChunk - 1) / kMomChunk; }
 
 // Moment sums, the read-out and the normalisation, enqueued on the run's stream.
@@ -987,8 +1010,8 @@ static rms_status finalize_impl(rms_run_handle *r)
     const WalkerState<Real> st = run_desc<Real>(r).st;
     if (q->n_rec > 0) {
         const int32_t nmc = mom_chunks(r->n_blocks);
-        moments_chunk_kernel<<<(unsigned)((int64_t)q->n_rec * nmc), 256, 0, s>>>(r->d_mom_partial, r->n_blocks, nmc,
-                                                                              r->d_mom_chunk);
+        moments_chunk_kernel<<<(unsigned)((int64_t)q->n_rec * nmc), 256, 0, s>>>(r->d_mom_partial, r->n_blocks, mom_sub(r),
+                                                                              nmc, r->d_mom_chunk);
         moments_reduce_kernel<<<(q->n_rec * kMoments + 127) / 128, 128, 0, s>>>(r->d_mom_chunk, q->n_rec, nmc,
                                                                                 r->d_mom);
         RMS_CUDA(cudaGetLastError());
@@ -1083,7 +1106,7 @@ rms_status rms::run_setup(rms_run_handle *r, bool with_cancel_and_events)
         RMS_CUDA(cudaMallocAsync((void **)&r->d_sort, morton_scratch_bytes(r->W), s));
         morton_plan(q->sub->nx, q->sub->ny, q->sub->nz, &r->sort_shift, &r->sort_passes);
     }
-    const size_t nmp = (size_t)std::max(q->n_rec, 1) * r->n_blocks * kMoments;
+    const size_t nmp = (size_t)std::max(q->n_rec, 1) * r->n_blocks * mom_sub(r) * kMoments;
     RMS_CUDA(cudaMallocAsync((void **)&r->d_mom_partial, sizeof(double) * nmp, s));
     // zero: a run that ends before some recording steps reports zero sums for them
     RMS_CUDA(cudaMemsetAsync(r->d_mom_partial, 0, sizeof(double) * nmp, s));
@@ -1184,8 +1207,8 @@ static rms_status run_import(rms_run_handle *r, const rms_run_state *from)
     if (from->moments)
         for (int rr = 0; rr < q->n_rec; ++rr)
             if (q->rec_steps[rr] <= from->step)
-                RMS_CUDA(cudaMemcpyAsync(r->d_mom_partial + (size_t)rr * r->n_blocks * kMoments, from->moments + 22 * rr,
-                                         sizeof(double) * kMoments, cudaMemcpyHostToDevice, s));
+                RMS_CUDA(cudaMemcpyAsync(r->d_mom_partial + (size_t)rr * r->n_blocks * mom_sub(r) * kMoments,
+                                         from->moments + 22 * rr, sizeof(double) * kMoments, cudaMemcpyHostToDevice, s));
     void *tmp[] = {d_i, d_i0, d_c, d_o, d_o0, d_A, d_ph, d_h};
     for (void *x : tmp)
         if (x) RMS_CUDA(cudaFreeAsync(x, s));
@@ -1247,6 +1270,8 @@ extern "C" rms_status rms_run_range(rms_sequence *q, const rms_run_desc *d, cons
     r->flags = d->flags;
     r->interaction = d->interaction;
     r->stream = (cudaStream_t)d->stream;
+    r->quad = r->precision == RMS_FP64 && r->interaction == RMS_EC && q->sub->rho.empty() &&
+              (r->flags & kVerifyFlags) == 0 && r->W <= kQuadMaxWalkers;
     int32_t spl = d->steps_per_launch;
     if (spl == 0) {
         // about 2e9 walker-steps per launch (a few tens of ms); 8e9 with Morton

@@ -74,6 +74,7 @@ struct rms_run_handle {
     int32_t interaction = RMS_EC;
     cudaStream_t stream = nullptr;
     int32_t n_blocks = 0;
+    bool quad = false;  // four lanes to a walker (walk_quad.cuh); moment partials per 32 walkers
     char *d_state = nullptr;  // one allocation for the walker state
     rms::WalkerState<double> st64{};
     rms::WalkerState<float> st32{};

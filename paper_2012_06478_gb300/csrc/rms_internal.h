@@ -30,6 +30,12 @@ RMS_EXTERN_LAUNCH_WALK(float, kInteractRS, true)
 RMS_EXTERN_LAUNCH_WALK(float, kInteractERL, true)
 #undef RMS_EXTERN_LAUNCH_WALK
 
+// The plain form's elastic collision with four lanes to a walker (walk_quad.cuh):
+// the moments' partials are per 32 walkers, four to a block of the others.
+cudaError_t launch_walk_quad(int n_shapes, cudaStream_t stream, const Geometry &g, const Tables<double> &t,
+                             const WalkerState<double> &st, const RunCtl &ctl, int64_t k_begin, int64_t k_end,
+                             int32_t rec);
+
 template <typename Real>
 cudaError_t launch_walk_batched(int ns_bucket, int32_t n_tasks, cudaStream_t stream, const ReqDesc<Real> *reqs,
                                 const BlockTask *tasks);
