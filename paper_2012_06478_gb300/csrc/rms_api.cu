@@ -19,6 +19,7 @@
 #include "rms_device.cuh"
 #include "rms_handles.h"
 #include "rms_internal.h"
+#include "serial_sum.cuh"
 
 using namespace rms;
 
@@ -263,14 +264,13 @@ __device__ __forceinline__ void neumaier(double &sum, double &comp, double x)
 // the same to the bit.
 //
 // What bounds it: three chains of N dependent additions (F, the sum, its
-// compensation), each one FP64 latency a step.  One thread doing all of a
-// step's operations -- two products and six or seven additions, each of which
-// holds GB300's narrow FP64 pipe as long as a whole warp's would -- was most of
-// a set-up: substrate, sequence of 6 shapes of 1e5 steps and a first run of 200
-// steps took 35.1 ms.  Here the chains run in three warps at once, each a chunk
-// behind the one before it, with only their own addition; the products F^2 and
-// dt G and the corrections, which no chain feeds back into, are done by all
-// threads between: 8.2 ms for the same calls.
+// compensation).  One thread doing all of a step's operations took most of a
+// set-up: substrate, sequence of 6 shapes of 1e5 steps and a first run of 200
+// steps in 35.1 ms.  Here the chains run in three warps at once, each a chunk
+// behind the one before it; the products F^2 and dt G and the corrections,
+// which no chain feeds back into, are done by all threads between (5.69 ms with
+// one addition after another, 8.2 ms for the calls).  Each chain takes 32 steps
+// at a time (serial_sum.cuh): 4.9 ms for the calls.
 constexpr int kBvThreads = 256;
 constexpr int kBvChunk = 1024;
 
@@ -285,7 +285,7 @@ __global__ void __launch_bounds__(kBvThreads) bvalue_kernel(int64_t N, int32_t S
     const double *g = G + (int64_t)s * N;
     const int chunks = (int)((N + kBvChunk - 1) / kBvChunk);
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    double chain = 0.0;  // lane 0 of warp 0: F; of warp 1: the sum; of warp 2: its compensation
+    double carry = 0.0;  // warp 0: F; warp 1: the sum; warp 2: its compensation
     for (int it = 0; it < chunks + 2; ++it) {
         double *const b0 = buf[it % 3], *const b1 = buf[(it + 2) % 3], *const b2 = buf[(it + 1) % 3];
         const auto length = [&](int c) {  // steps of chunk c (0: no such chunk)
@@ -303,20 +303,27 @@ __global__ void __launch_bounds__(kBvThreads) bvalue_kernel(int64_t N, int32_t S
             }
         }
         __syncthreads();
-        if (lane == 0 && warp < 3) {
-            if (warp == 0) {
-#pragma unroll 8
-                for (int i = 0; i < n0; ++i) {
-                    const double w = b0[i];
-                    b0[i] = chain;
-                    chain = chain + w;
+        if (warp < 3) {
+            double *const x = warp == 0 ? b0 : (warp == 1 ? b1 : b2);
+            const int n = warp == 0 ? n0 : (warp == 1 ? n1 : n2);
+            if (warp == 1 && lane == 0) t1[0] = carry;
+            for (int i = 0; i < n; i += 32) {
+                const int m = min(32, n - i);
+                double after = 0.0;
+                const double before = carry;
+                carry = chain::serial_sums(carry, lane < m ? x[i + lane] : 0.0, m, after);
+                if (warp == 0) {  // F before each step
+                    const double last = __shfl_up_sync(0xffffffffu, after, 1);
+                    if (lane < m) x[i + lane] = lane == 0 ? before : last;
+                } else if (warp == 1) {
+                    if (lane < m) t1[i + lane + 1] = after;
                 }
             }
         }
         __syncthreads();
     }
     __shared__ double total[2];
-    if (lane == 0 && (warp == 1 || warp == 2)) total[warp - 1] = chain;
+    if (lane == 0 && (warp == 1 || warp == 2)) total[warp - 1] = carry;
     __syncthreads();
     const double bs = dt * (total[0] + total[1]);
     if (threadIdx.x == 0) bs_out[s] = bs;
