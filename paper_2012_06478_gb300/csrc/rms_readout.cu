@@ -8,6 +8,7 @@
 
 #include <algorithm>
 
+#include "f32x2.cuh"
 #include "rms_internal.h"
 #include "rms_readout.cuh"
 
@@ -56,31 +57,6 @@ __device__ __forceinline__ int top_exponent(double a, double b)
     const unsigned u = (unsigned)(fix::double_word(a) >> 32) & 0x7FFFFFFFu;
     const unsigned v = (unsigned)(fix::double_word(b) >> 32) & 0x7FFFFFFFu;
     return (int)(__reduce_max_sync(0xffffffffu, max(u, v)) >> 20);
-}
-
-// Two single-precision numbers at a time (Blackwell's packed operations).
-struct F2 {
-    uint64_t v;
-};
-__device__ __forceinline__ F2 pair_of(float x, float y)
-{
-    F2 r;
-    asm("mov.b64 %0, {%1, %2};" : "=l"(r.v) : "f"(x), "f"(y));
-    return r;
-}
-__device__ __forceinline__ float first(F2 a) { return __uint_as_float((uint32_t)a.v); }
-__device__ __forceinline__ float second(F2 a) { return __uint_as_float((uint32_t)(a.v >> 32)); }
-__device__ __forceinline__ F2 operator+(F2 a, F2 b)
-{
-    F2 r;
-    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r.v) : "l"(a.v), "l"(b.v));
-    return r;
-}
-__device__ __forceinline__ F2 operator-(F2 a, F2 b)
-{
-    F2 r;
-    asm("sub.rn.f32x2 %0, %1, %2;" : "=l"(r.v) : "l"(a.v), "l"(b.v));
-    return r;
 }
 
 // Sums of at most 64 pairs of numbers below 1: each is split at 2^-16 and 2^-33

@@ -26,6 +26,7 @@
 #include <cstdint>
 #include <type_traits>
 
+#include "f32x2.cuh"
 #include "rms_device.cuh"
 #include "soft_fp64.cuh"
 
@@ -294,6 +295,108 @@ __device__ __forceinline__ void kahan_add(Real &sum, Real &comp, Real x)
     sum = t;
 }
 
+// The phases of NS shapes by axis, component k = 3 shape + axis, with the FP32
+// form's Kahan compensations.
+template <typename Real, int NS>
+struct Phases {
+    Real p[3 * NS];
+    __device__ __forceinline__ void load(const WalkerState<Real> &st, int n, int64_t W, int64_t li)
+    {
+#pragma unroll
+        for (int k = 0; k < 3 * NS; ++k) p[k] = k < 3 * n ? st.phase[k * W + li] : Real(0);
+    }
+    __device__ __forceinline__ void store(const WalkerState<Real> &st, int n, int64_t W, int64_t li) const
+    {
+#pragma unroll
+        for (int k = 0; k < 3 * NS; ++k)
+            if (k < 3 * n) st.phase[k * W + li] = p[k];
+    }
+    // p += w dx for shape s
+    template <typename Weight>
+    __device__ __forceinline__ void add(int n, const Real dx[3], Weight weight)
+    {
+#pragma unroll
+        for (int s = 0; s < NS; ++s)
+            if (s < n) {
+                const Real w = weight(s);
+#pragma unroll
+                for (int a = 0; a < 3; ++a) p[3 * s + a] = p[3 * s + a] + mulr(w, dx[a]);
+            }
+    }
+};
+// FP32: two components an instruction (x and y of a shape, or the six of two
+// shapes), the additions that bound a step of several shapes.  The
+// compensation is kept negated, so that y = w dx - c is one multiply-add.
+template <int NS>
+struct Phases<float, NS> {
+    static constexpr int kPairs = 3 * NS / 2;  // and, of an odd number of shapes, the last z
+    F2 p[kPairs], nc[kPairs];
+    float pz, ncz;
+    __device__ __forceinline__ void load(const WalkerState<float> &st, int n, int64_t W, int64_t li)
+    {
+        const auto of = [&](const float *from, int k) { return k < 3 * n ? from[k * W + li] : 0.0f; };
+#pragma unroll
+        for (int k = 0; k < kPairs; ++k) {
+            p[k] = pair_of(of(st.phase, 2 * k), of(st.phase, 2 * k + 1));
+            nc[k] = pair_of(-of(st.phase_c, 2 * k), -of(st.phase_c, 2 * k + 1));
+        }
+        pz = ncz = 0.0f;
+        if (NS & 1) {
+            pz = of(st.phase, 3 * NS - 1);
+            ncz = -of(st.phase_c, 3 * NS - 1);
+        }
+    }
+    __device__ __forceinline__ void store(const WalkerState<float> &st, int n, int64_t W, int64_t li) const
+    {
+        const auto put = [&](int k, float x, float c) {
+            if (k < 3 * n) {
+                st.phase[k * W + li] = x;
+                st.phase_c[k * W + li] = -c;
+            }
+        };
+#pragma unroll
+        for (int k = 0; k < kPairs; ++k) {
+            put(2 * k, first(p[k]), first(nc[k]));
+            put(2 * k + 1, second(p[k]), second(nc[k]));
+        }
+        if (NS & 1) put(3 * NS - 1, pz, ncz);
+    }
+    template <int K>
+    __device__ __forceinline__ void add_pair(F2 w, F2 dx)
+    {
+        static_assert(K < kPairs, "a pair of this many shapes");
+        const F2 y = fma2(w, dx, nc[K]), t = p[K] + y;
+        nc[K] = y - (t - p[K]);
+        p[K] = t;
+    }
+    // shapes s and s + 1; the last of an odd number alone
+    template <int S, typename Weight>
+    __device__ __forceinline__ void add_from(int n, F2 xy, F2 zx, F2 yz, float z, Weight weight)
+    {
+        if constexpr (S < NS) {
+            if (S >= n) return;
+            const float w0 = weight(S);
+            add_pair<3 * S / 2>(pair_of(w0, w0), xy);
+            if constexpr (S + 1 < NS) {
+                // a shape beyond the last adds w = 0 to phases that nobody reads
+                const float w1 = S + 1 < n ? weight(S + 1) : 0.0f;
+                add_pair<3 * S / 2 + 1>(pair_of(w0, w1), zx);
+                add_pair<3 * S / 2 + 2>(pair_of(w1, w1), yz);
+                add_from<S + 2>(n, xy, zx, yz, z, weight);
+            } else {
+                const float y = fmaf(w0, z, ncz), t = pz + y;
+                ncz = y - (t - pz);
+                pz = t;
+            }
+        }
+    }
+    template <typename Weight>
+    __device__ __forceinline__ void add(int n, const float dx[3], Weight weight)
+    {
+        add_from<0>(n, pair_of(dx[0], dx[1]), pair_of(dx[2], dx[0]), pair_of(dx[1], dx[2]), dx[2], weight);
+    }
+};
+
 // The 22 moment terms at a recording step (Sec. 2.3, narrow-pulse D and K):
 // alpha, alpha dx_i dx_j (i <= j), alpha dx_i dx_j dx_k dx_l (i<=j<=k<=l),
 // each reduced over the warp as soon as it is formed (few live registers);
@@ -337,9 +440,8 @@ __device__ __forceinline__ void warp_moments(double al, const double dx[3], doub
 // absorbing membranes (Sec. 2.1.3, magnetization transfer; t.Tmt non-null).
 // RELAX: 1 some label has a finite T1 or T2, 0 none has (every rate is 0, the
 // exponent keeps its start value and Eq. 5 drops out), 2 decided at run time.
-// RK: draw with the round keys of ctl.rk, computed once on the host (no key
-// schedule per draw: 2.4 % faster on the FP32 step); otherwise advance the
-// key from ctl.seed in every draw (the batched kernel, whose request
+// RK: hold the round keys of ctl.rk (computed once on the host) for the slice;
+// otherwise read them at every draw (the batched kernel, whose request
 // descriptors sit in shared memory).  `rec` is the first recording step's
 // index beyond k_begin.
 template <typename Real, int NS, bool HASH, int IM, bool MT, int RELAX, bool RK = false>
@@ -357,9 +459,11 @@ __device__ __forceinline__ void walk_block(const Geometry &g, const Tables<Real>
     // the round keys, loop-invariant and warp-uniform: read once here (read
     // from the launch parameters inside the step loop they took 16 constant
     // loads per warp-step; hoisted, the step is 1.3 % faster)
-    uint32_t rk[kRoundKeys];
+    [[maybe_unused]] uint32_t rk[kRoundKeys];
+    if constexpr (RK) {
 #pragma unroll
-    for (int i = 0; i < kRoundKeys; ++i) rk[i] = ctl.rk[i];
+        for (int i = 0; i < kRoundKeys; ++i) rk[i] = ctl.rk[i];
+    }
     // threads beyond the last walker walk a copy of it and write nothing: no
     // branch on it in the step loop
     const bool active = block * kWalkBlock + threadIdx.x < ctl.n_walkers;
@@ -394,15 +498,8 @@ __device__ __forceinline__ void walk_block(const Geometry &g, const Tables<Real>
     Real sc = __ldg(t.s + c);  // step length of label c
     Real A = st.A[li], Ac = Real(0);
     if constexpr (!kF64) Ac = st.A_c[li];
-    Real ph[NS][3], phc[NS][3];
-#pragma unroll
-    for (int s = 0; s < NS; ++s)
-#pragma unroll
-        for (int a = 0; a < 3; ++a) {
-            ph[s][a] = s < ctl.n_shapes ? st.phase[((int64_t)s * 3 + a) * ctl.n_walkers + li] : Real(0);
-            phc[s][a] =
-                (!kF64 && s < ctl.n_shapes) ? st.phase_c[((int64_t)s * 3 + a) * ctl.n_walkers + li] : Real(0);
-        }
+    Phases<Real, NS> ph;
+    ph.load(st, ctl.n_shapes, ctl.n_walkers, li);
     [[maybe_unused]] uint64_t h = 0;
     // face events, crossings into another label, reflections (verification kernel)
     [[maybe_unused]] int32_t nev = 0, ncr = 0, nrf = 0;
@@ -464,7 +561,7 @@ __device__ __forceinline__ void walk_block(const Geometry &g, const Tables<Real>
             if constexpr (RK)
                 x = philox4x32_10_rk(U4{(uint32_t)w, (uint32_t)(w >> 32), (uint32_t)k, (kTagDir << 16) | att}, rk);
             else
-                x = draw(ctl.seed, w, (uint32_t)k, kTagDir, att);
+                x = philox4x32_10_rk(U4{(uint32_t)w, (uint32_t)(w >> 32), (uint32_t)k, (kTagDir << 16) | att}, ctl.rk);
             Real n[3];
             direction_from(x.x, x.y, t.trig, n);
             // ---- face walk (Sec. 2.2 items 3-4)
@@ -753,19 +850,8 @@ __device__ __forceinline__ void walk_block(const Geometry &g, const Tables<Real>
             Real dx[3];
 #pragma unroll
             for (int a = 0; a < 3; ++a) dx[a] = mulr(lp, (Real)di[a] + (o[a] - o0[a]));
-#pragma unroll
-            for (int s = 0; s < NS; ++s) {
-                if (s < ctl.n_shapes) {
-                    const Real wgs = NS == 1 ? wg : __ldg(t.wG + (int64_t)s * t.pitch + (k - 1));
-#pragma unroll
-                    for (int a = 0; a < 3; ++a) {
-                        if (kF64)
-                            ph[s][a] = ph[s][a] + dmul(wgs, dx[a]);
-                        else
-                            kahan_add(ph[s][a], phc[s][a], wgs * dx[a]);
-                    }
-                }
-            }
+            ph.add(ctl.n_shapes, dx,
+                   [&](int s) { return NS == 1 ? wg : __ldg(t.wG + (int64_t)s * t.pitch + (k - 1)); });
         }
         // ---- displacement moments at recording steps (block-uniform branch)
         if (k == next_rec) {
@@ -799,14 +885,7 @@ __device__ __forceinline__ void walk_block(const Geometry &g, const Tables<Real>
         st.c[li] = c;
         st.A[li] = A;
         if (!kF64) st.A_c[li] = Ac;
-#pragma unroll
-        for (int s = 0; s < NS; ++s)
-            if (s < ctl.n_shapes)
-#pragma unroll
-                for (int a = 0; a < 3; ++a) {
-                    st.phase[((int64_t)s * 3 + a) * ctl.n_walkers + li] = ph[s][a];
-                    if (!kF64) st.phase_c[((int64_t)s * 3 + a) * ctl.n_walkers + li] = phc[s][a];
-                }
+        ph.store(st, ctl.n_shapes, ctl.n_walkers, li);
         if constexpr (HASH) {
             st.hash[li] = h;
             if (st.counts) {
@@ -822,21 +901,25 @@ __device__ __forceinline__ void walk_block(const Geometry &g, const Tables<Real>
 // the compiler's choice).  The plain form's one-shape kernel: its integer-ALU
 // arithmetic is made of long dependent chains, whose latency more warps hide,
 // and 5 blocks (at most 102 registers) measured 6 % faster than the
-// unconstrained 4.  The FP32 form's one-shape elastic-collision kernel: 8
-// blocks (64 registers, 32 warps per SM), 21.8 ms for 1e6 walkers x 2000 steps
-// on 200x200x400 axons against 22.0 ms at 9 (56 registers, small spills) and
-// 22.5 ms at 7.  The RS/ERL and absorbing-membrane kernels would spill under
-// such bounds, and kernels with more shapes keep the registers their phases
-// need.
+// unconstrained 4.  The FP32 form's elastic-collision kernels: as many blocks
+// as their phases leave registers for without spills -- one shape 8 (64
+// registers: 21.8 ms for 1e6 walkers x 2000 steps on 200x200x400 axons against
+// 22.0 ms at 9 with small spills and 22.5 ms at 7; absorbing membranes, 3e5
+// walkers x 3000 steps, 14.7 ms against 16.6 at 5), six shapes 5 (4e6 walkers x
+// 1000 steps 75 ms against 88 with the kernel of eight at 4).  RS and ERL keep a
+// step's start beside the state and would spill at 8.
 template <typename Real, int NS, bool HASH, int IM, bool MT>
-constexpr int kWalkMinBlocks = (NS != 1) ? 0
-                               : std::is_same<Real, double>::value ? 5
-                               : (IM != kInteractEC || MT) ? 0
-                               : HASH ? 7 : 8;  // the verification kernel would spill at 8
+constexpr int walk_min_blocks()
+{
+    if (std::is_same<Real, double>::value) return NS == 1 ? 5 : 0;
+    if (HASH) return NS == 1 && IM == kInteractEC && !MT ? 7 : 0;  // the verification kernel would spill at 8
+    if (IM != kInteractEC) return NS == 1 && IM == kInteractRS && !MT ? 7 : 0;
+    return NS == 1 ? 8 : NS == 2 ? (MT ? 7 : 8) : NS == 3 ? 7 : NS == 4 ? 6 : NS == 6 ? 5 : 4;
+}
 
 // One run: block b of the grid advances walkers b*kWalkBlock ... of the run.
 template <typename Real, int NS, bool HASH, int IM, bool MT, int RELAX>
-__global__ void __launch_bounds__(kWalkBlock, kWalkMinBlocks<Real, NS, HASH, IM, MT>)
+__global__ void __launch_bounds__(kWalkBlock, (walk_min_blocks<Real, NS, HASH, IM, MT>()))
 walk_kernel(Geometry g, Tables<Real> t, WalkerState<Real> st, RunCtl ctl, int64_t k_begin, int64_t k_end, int32_t rec)
 {
     walk_block<Real, NS, HASH, IM, MT, RELAX, true>(g, t, st, ctl, blockIdx.x, k_begin, k_end, rec);
@@ -846,7 +929,7 @@ walk_kernel(Geometry g, Tables<Real> t, WalkerState<Real> st, RunCtl ctl, int64_
 // a block of walkers of one request for that request's next steps.  The
 // request descriptors and the task table are read once per block.
 template <typename Real, int NS>
-__global__ void __launch_bounds__(kWalkBlock, (std::is_same<Real, float>::value && NS <= 2) ? 8 : 4)
+__global__ void __launch_bounds__(kWalkBlock, std::is_same<Real, double>::value || NS > 4 ? 4 : NS > 2 ? 6 : 8)
 walk_batched_kernel(const ReqDesc<Real> *reqs, const BlockTask *tasks, int32_t n_tasks)
 {
     if ((int32_t)blockIdx.x >= n_tasks) return;
@@ -908,20 +991,26 @@ cudaError_t launch_walk(int n_shapes, bool hash, dim3 grid, cudaStream_t stream,
 #define RMS_LAUNCH(NSV, HASHV, RELAXV)                                                                     \
     walk_kernel<Real, NSV, HASHV, IM, MT, RELAXV><<<grid, kWalkBlock, 0, stream>>>(g, t, st, ctl, k_begin, \
                                                                                   k_end, rec)
-#define RMS_LAUNCH_NS(HASHV, RELAXV)    \
-    do {                                \
-        if (n_shapes <= 1)              \
-            RMS_LAUNCH(1, HASHV, RELAXV); \
-        else if (n_shapes <= 2)         \
-            RMS_LAUNCH(2, HASHV, RELAXV); \
-        else if (n_shapes <= 4)         \
-            RMS_LAUNCH(4, HASHV, RELAXV); \
-        else                            \
-            RMS_LAUNCH(8, HASHV, RELAXV); \
+// kernels of three and six shapes where they pay: the FP32 form's elastic collision
+#define RMS_LAUNCH_NS(HASHV, RELAXV)                                                  \
+    do {                                                                              \
+        constexpr bool kMore = !std::is_same<Real, double>::value && IM == kInteractEC && !MT && !HASHV; \
+        if (n_shapes <= 1)                                                            \
+            RMS_LAUNCH(1, HASHV, RELAXV);                                             \
+        else if (n_shapes <= 2)                                                       \
+            RMS_LAUNCH(2, HASHV, RELAXV);                                             \
+        else if (kMore && n_shapes <= 3)                                              \
+            RMS_LAUNCH(kMore ? 3 : 4, HASHV, RELAXV);                                 \
+        else if (n_shapes <= 4)                                                       \
+            RMS_LAUNCH(4, HASHV, RELAXV);                                             \
+        else if (kMore && n_shapes <= 6)                                              \
+            RMS_LAUNCH(kMore ? 6 : 8, HASHV, RELAXV);                                 \
+        else                                                                          \
+            RMS_LAUNCH(8, HASHV, RELAXV);                                             \
     } while (0)
     if (hash)
         RMS_LAUNCH_NS(true, 2);
-    else if constexpr (IM != kInteractEC || MT)
+    else if constexpr (IM != kInteractEC)
         RMS_LAUNCH_NS(false, 2);
     else if (t.any_relax)
         RMS_LAUNCH_NS(false, 1);
