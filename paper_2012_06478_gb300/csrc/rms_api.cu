@@ -995,12 +995,11 @@ rms_status rms::run_walk(rms_run_handle *r, int64_t k0, int64_t k1)
     return r->precision == RMS_FP32 ? walk_impl<float>(r, k0, k1) : walk_impl<double>(r, k0, k1);
 }
 
-// Plain-form runs of at most this many walkers take four lanes to a walker: two
-// waves of its blocks (five of 32 walkers an SM).  600 steps of 500, 1e4, 2e4 and
-// 4e4 walkers in axons: 1.95, 2.39, 3.12 and 5.14 ms against 4.41, 4.52, 5.31 and
-// 6.46; with relaxation and unequal D 2.09, 2.62, 3.47 and 5.71 against 4.45,
-// 4.59, 5.42 and 6.54.  In a third wave the one-thread kernel's fewer
-// instructions win (5e4: 6.98 against 6.75).
+// Plain-form runs of at most this many walkers take four lanes to a walker.  600
+// steps of 5000, 1e4, 2e4 and 4e4 walkers in axons: 2.2, 2.4, 3.2 and 5.1 ms
+// against 4.5, 4.5, 5.2 and 6.0; with relaxation and unequal D 2.3, 2.6, 3.5 and
+// 5.8 against 4.5, 4.5, 5.2 and 6.2.  Above, the one-thread kernel's fewer
+// instructions win (3001 steps of 50 001 with relaxation: 28.5 against 30.7).
 constexpr int64_t kQuadMaxWalkers = 2 * 5 * 152 * 32;
 
 // Moment partials of a block of the walk.

@@ -153,6 +153,8 @@ __device__ __forceinline__ double u64_scaled_rn(unsigned long long N)
     return __longlong_as_double((long long)(((unsigned long long)(e + 1023) << 52) | (q & 0x000FFFFFFFFFFFFFULL)));
 }
 
+// UNROLL: all products side by side (the four-lane kernel, bound by their latency).
+template <bool UNROLL = false>
 __device__ __forceinline__ void direction_from(uint32_t x0, uint32_t x1, const double *__restrict__ trig,
                                                double n[3])
 {
@@ -184,12 +186,29 @@ __device__ __forceinline__ void direction_from(uint32_t x0, uint32_t x1, const d
     const double se = e + mul_normal(mul_normal(e, t), -1.0 / 6.0 + mul_normal(t, 1.0 / 120.0));
     const double ce = 1.0 + mul_normal(t, -1.0 / 2.0 + mul_normal(t, 1.0 / 24.0));
     const double cj = __ldg(trig + 2 * j), sj = __ldg(trig + 2 * j + 1);
-    const double cs = mul_normal(cj, ce) - mul_normal(sj, se);
-    const double sn = mul_normal(sj, ce) + mul_normal(cj, se);
+    // cs = cj ce - sj se, then sn = sj ce - (-cj) se
+    double cs = 0.0, sn = 0.0;
+    {
+        double p = cj, q = sj;
+#pragma unroll UNROLL ? 2 : 1
+        for (int i = 0; i < 2; ++i) {
+            cs = sn;
+            sn = mul_normal(p, ce) - mul_normal(q, se);
+            const double m = -p;
+            p = q;
+            q = m;
+        }
+    }
     double cx, sy;
     octant_map(oct, cs, sn, cx, sy);
-    n[0] = mul_normal(r, cx);
-    n[1] = mul_normal(r, sy);
+#pragma unroll UNROLL ? 2 : 1
+    for (int i = 0; i < 2; ++i) {
+        const double x = mul_normal(r, cx);
+        cx = sy;
+        sy = x;
+    }
+    n[0] = cx;
+    n[1] = sy;
     n[2] = z;
 }
 
@@ -233,6 +252,23 @@ __device__ __forceinline__ void direction_from(uint32_t x0, uint32_t x1, const d
     n[0] = r * (negx ? -a : a);
     n[1] = r * (negy ? -b : b);
     n[2] = z;
+}
+
+// The plain form's loops over axes are not unrolled: its integer-ALU products
+// and quotients are 30 to 150 instructions each, and with three copies of each
+// the step's code was larger than the instruction caches (instruction fetch the
+// first of the stalls): 3.3e5 walkers x 3000 steps 139 ms unrolled, 120 with the
+// loops, 112.5 with the phases and start offsets in shared memory too, the
+// offsets of an event's other two axes moved in one loop and 6 blocks an SM.
+// Axis r is in slot 0 in the loop's turn r; after three turns every axis is back
+// in its own.
+template <typename T>
+__device__ __forceinline__ void rotate(T x[3])
+{
+    const T t = x[0];
+    x[0] = x[1];
+    x[1] = x[2];
+    x[2] = t;
 }
 
 // Saturation (Sec. 2.1.3): A = +inf (FP64 form) or kSaturatedF (FP32 form).
@@ -295,33 +331,40 @@ __device__ __forceinline__ void kahan_add(Real &sum, Real &comp, Real x)
     sum = t;
 }
 
-// The phases of NS shapes by axis, component k = 3 shape + axis, with the FP32
-// form's Kahan compensations.
+// The phases of NS shapes by axis, component k = 3 shape + axis.  Plain form: in
+// shared memory, with the start offsets, so that loops over axes and shapes need
+// not be unrolled and the registers hold more warps.
 template <typename Real, int NS>
 struct Phases {
-    Real p[3 * NS];
+    double *p, *start;  // [component or axis][thread]
+    // shared memory of a block
+    static size_t bytes(int n) { return sizeof(double) * (3 * n + 3) * kWalkBlock; }
     __device__ __forceinline__ void load(const WalkerState<Real> &st, int n, int64_t W, int64_t li)
     {
+        extern __shared__ double s_axes[];
+        start = s_axes + threadIdx.x;
+        p = start + 3 * kWalkBlock;
+        for (int k = 0; k < 3 * n; ++k) p[k * kWalkBlock] = st.phase[k * W + li];
 #pragma unroll
-        for (int k = 0; k < 3 * NS; ++k) p[k] = k < 3 * n ? st.phase[k * W + li] : Real(0);
+        for (int a = 0; a < 3; ++a) start[a * kWalkBlock] = st.o0[a][li];
     }
     __device__ __forceinline__ void store(const WalkerState<Real> &st, int n, int64_t W, int64_t li) const
     {
-#pragma unroll
-        for (int k = 0; k < 3 * NS; ++k)
-            if (k < 3 * n) st.phase[k * W + li] = p[k];
+        for (int k = 0; k < 3 * n; ++k) st.phase[k * W + li] = p[k * kWalkBlock];
     }
-    // p += w dx for shape s
+    // component `axis` of every shape's phase += w dx
     template <typename Weight>
-    __device__ __forceinline__ void add(int n, const Real dx[3], Weight weight)
+    __device__ __forceinline__ void add(int n, int axis, double dx, Weight weight)
     {
-#pragma unroll
-        for (int s = 0; s < NS; ++s)
-            if (s < n) {
-                const Real w = weight(s);
-#pragma unroll
-                for (int a = 0; a < 3; ++a) p[3 * s + a] = p[3 * s + a] + mulr(w, dx[a]);
+        if constexpr (NS == 1) {
+            p[axis * kWalkBlock] = p[axis * kWalkBlock] + dmul(weight(0), dx);
+        } else {
+#pragma unroll 1
+            for (int s = 0; s < n; ++s) {
+                double &x = p[(3 * s + axis) * kWalkBlock];
+                x = x + dmul(weight(s), dx);
             }
+        }
     }
 };
 // FP32: two components an instruction (x and y of a shape, or the six of two
@@ -332,6 +375,7 @@ struct Phases<float, NS> {
     static constexpr int kPairs = 3 * NS / 2;  // and, of an odd number of shapes, the last z
     F2 p[kPairs], nc[kPairs];
     float pz, ncz;
+    static size_t bytes(int) { return 0; }
     __device__ __forceinline__ void load(const WalkerState<float> &st, int n, int64_t W, int64_t li)
     {
         const auto of = [&](const float *from, int k) { return k < 3 * n ? from[k * W + li] : 0.0f; };
@@ -483,13 +527,14 @@ __device__ __forceinline__ void walk_block(const Geometry &g, const Tables<Real>
     else
         lp = g.voxel_f;
 
-    Real o[3], o0[3];
+    Real o[3];
+    [[maybe_unused]] Real o0[3];  // FP32 form; the plain form's are beside its phases
     int32_t di[3];
     int32_t v = 0;
 #pragma unroll
     for (int a = 0; a < 3; ++a) {
         o[a] = st.o[a][li];
-        o0[a] = st.o0[a][li];
+        if constexpr (!kF64) o0[a] = st.o0[a][li];
         di[a] = st.di[a][li];
         v += stride[a] * wrapped(st.i0[a][li] + di[a], N[a]);
     }
@@ -568,7 +613,11 @@ __device__ __forceinline__ void walk_block(const Geometry &g, const Tables<Real>
             Real rate = Real(0);
             if (relax) rate = __ldg(t.dtR + mode * L + c);
             [[maybe_unused]] const Real rate0 = rate;
-            Real d[3] = {mulr(n[0], sc), mulr(n[1], sc), mulr(n[2], sc)};
+            Real d[3] = {};
+            if constexpr (!kF64) {
+#pragma unroll
+                for (int a = 0; a < 3; ++a) d[a] = n[a] * sc;
+            }
             [[maybe_unused]] bool refused = false;
             // A face event on axis `best` moving up/down: where the voxel's own face
             // bits say that the voxel across is inside the volume and carries the same
@@ -633,12 +682,18 @@ __device__ __forceinline__ void walk_block(const Geometry &g, const Tables<Real>
                 // one division per axis: (1 - o)/d moving up, o/(-d) moving down, on the
                 // integer ALU (the IEEE quotient; the hardware division only for operands
                 // outside its range, e.g. o = -0)
-                double T[3];
-#pragma unroll
-                for (int a = 0; a < 3; ++a) {
-                    const double num = dgt0(d[a]) ? 1.0 - o[a] : o[a];
-                    const double den = __longlong_as_double(dbits(d[a]) & 0x7FFFFFFFFFFFFFFFLL);  // |d|
-                    T[a] = (dgt0(d[a]) || dlt0(d[a])) ? ddiv_nn(num, den) : kInf;
+                double T[3] = {};
+                const auto face_time = [](double o, double d) {
+                    return ddiv_nn(dgt0(d) ? 1.0 - o : o, __longlong_as_double(dbits(d) & 0x7FFFFFFFFFFFFFFFLL));
+                };
+#pragma unroll 1
+                for (int r = 0; r < 3; ++r) {
+                    d[0] = dmul(n[0], sc);
+                    T[0] = (dgt0(d[0]) || dlt0(d[0])) ? face_time(o[0], d[0]) : kInf;
+                    rotate(n);
+                    rotate(o);
+                    rotate(d);
+                    rotate(T);
                 }
                 double tau = 0.0;
                 // not unrolled in the plain form: its event pass carries the integer-ALU
@@ -662,18 +717,31 @@ __device__ __forceinline__ void walk_block(const Geometry &g, const Tables<Real>
                     if (relax) A = A + dmul(dts, rate);
                     tau = tmin;
                     if constexpr (HASH) ++nev;
-                    bool up = false;
-#pragma unroll
-                    for (int a = 0; a < 3; ++a) {
-                        if (a == best) {
-                            up = dgt0(d[a]);
-                            T[a] = kInf;
-                            o[a] = up ? 0.0 : 1.0;
-                            di[a] += up ? 1 : -1;
-                        } else {
-                            o[a] = dclamp01(o[a] + dmul(dts, d[a]));
+                    const bool up = dgt0(best == 2 ? d[2] : (best == 1 ? d[1] : d[0]));
+                    {
+                        // the two axes that meet no face move on: their offsets and steps,
+                        // taken out, moved in turn, and put back beside the face
+                        double oa = best == 0 ? o[1] : o[0], ob = best == 2 ? o[1] : o[2];
+                        double da = best == 0 ? d[1] : d[0], db = best == 2 ? d[1] : d[2];
+#pragma unroll 1
+                        for (int r = 0; r < 2; ++r) {
+                            const double x = dclamp01(oa + dmul(dts, da)), y = da;
+                            oa = ob;
+                            ob = x;
+                            da = db;
+                            db = y;
                         }
+                        const double face = up ? 0.0 : 1.0;
+                        o[0] = best == 0 ? face : oa;
+                        o[1] = best == 1 ? face : (best == 0 ? oa : ob);
+                        o[2] = best == 2 ? face : ob;
                     }
+#pragma unroll
+                    for (int a = 0; a < 3; ++a)
+                        if (a == best) {
+                            T[a] = kInf;
+                            di[a] += up ? 1 : -1;
+                        }
                     const int32_t sb = best == 2 ? stride[2] : (best == 1 ? stride[1] : 1);
                     const uint32_t bit = (best == 2 ? kFaceZ : (best == 1 ? kFaceY : kFaceX)) << (up ? 3 : 0);
                     int32_t nv = up ? v + sb : v - sb;
@@ -692,13 +760,14 @@ __device__ __forceinline__ void walk_block(const Geometry &g, const Tables<Real>
                             const double sn = __ldg(t.s + c);
                             if (dbits(sn) != dbits(sc)) {
                                 sc = sn;
-#pragma unroll
-                                for (int a = 0; a < 3; ++a) {
-                                    d[a] = dmul(n[a], sc);
-                                    if (dbits(T[a]) == 0x7FF0000000000000LL) continue;
-                                    const double num = dgt0(d[a]) ? 1.0 - o[a] : o[a];
-                                    T[a] = tau +
-                                           ddiv_nn(num, __longlong_as_double(dbits(d[a]) & 0x7FFFFFFFFFFFFFFFLL));
+#pragma unroll 1
+                                for (int r = 0; r < 3; ++r) {
+                                    d[0] = dmul(n[0], sc);
+                                    if (dbits(T[0]) != 0x7FF0000000000000LL) T[0] = tau + face_time(o[0], d[0]);
+                                    rotate(n);
+                                    rotate(o);
+                                    rotate(d);
+                                    rotate(T);
                                 }
                             }
                         }
@@ -711,8 +780,12 @@ __device__ __forceinline__ void walk_block(const Geometry &g, const Tables<Real>
                 }
                 if (IM == kInteractEC || !refused) {
                     const double rem = 1.0 - tau;
-#pragma unroll
-                    for (int a = 0; a < 3; ++a) o[a] = dclamp01(o[a] + dmul(rem, d[a]));
+#pragma unroll 1
+                    for (int r = 0; r < 3; ++r) {
+                        o[0] = dclamp01(o[0] + dmul(rem, d[0]));
+                        rotate(o);
+                        rotate(d);
+                    }
                     if (relax) A = A + dmul(rem, rate);
                 }
             } else {
@@ -847,18 +920,33 @@ __device__ __forceinline__ void walk_block(const Geometry &g, const Tables<Real>
         }
         // ---- phase (Eq. 7, right end point of each step)
         if (graded) {
-            Real dx[3];
+            const auto weight = [&](int s) { return NS == 1 ? wg : __ldg(t.wG + (int64_t)s * t.pitch + (k - 1)); };
+            if constexpr (kF64) {
+#pragma unroll 1
+                for (int r = 0; r < 3; ++r) {
+                    ph.add(ctl.n_shapes, r, dmul(lp, (double)di[0] + (o[0] - ph.start[r * kWalkBlock])), weight);
+                    rotate(o);
+                    rotate(di);
+                }
+            } else {
+                Real dx[3];
 #pragma unroll
-            for (int a = 0; a < 3; ++a) dx[a] = mulr(lp, (Real)di[a] + (o[a] - o0[a]));
-            ph.add(ctl.n_shapes, dx,
-                   [&](int s) { return NS == 1 ? wg : __ldg(t.wG + (int64_t)s * t.pitch + (k - 1)); });
+                for (int a = 0; a < 3; ++a) dx[a] = lp * ((Real)di[a] + (o[a] - o0[a]));
+                ph.add(ctl.n_shapes, dx, weight);
+            }
         }
         // ---- displacement moments at recording steps (block-uniform branch)
         if (k == next_rec) {
             double dx[3];
+            const auto start = [&](int a) -> double {
+                if constexpr (kF64)
+                    return ph.start[a * kWalkBlock];
+                else
+                    return (double)o0[a];
+            };
 #pragma unroll
             for (int a = 0; a < 3; ++a)
-                dx[a] = g.voxel_um * ((double)di[a] + ((double)o[a] - (double)o0[a]));
+                dx[a] = g.voxel_um * ((double)di[a] + ((double)o[a] - start(a)));
             double al = 1.0;  // alpha = exp(-A); mostly A = 0 without relaxation
             if (A != Real(0)) al = kF64 ? exp(-(double)A) : exp(-((double)A - (double)Ac));
             if (!active) al = 0.0;
@@ -898,20 +986,19 @@ __device__ __forceinline__ void walk_block(const Geometry &g, const Tables<Real>
 }
 
 // Resident blocks per SM the register allocation must allow (0: no bound,
-// the compiler's choice).  The plain form's one-shape kernel: its integer-ALU
-// arithmetic is made of long dependent chains, whose latency more warps hide,
-// and 5 blocks (at most 102 registers) measured 6 % faster than the
-// unconstrained 4.  The FP32 form's elastic-collision kernels: as many blocks
-// as their phases leave registers for without spills -- one shape 8 (64
-// registers: 21.8 ms for 1e6 walkers x 2000 steps on 200x200x400 axons against
-// 22.0 ms at 9 with small spills and 22.5 ms at 7; absorbing membranes, 3e5
-// walkers x 3000 steps, 14.7 ms against 16.6 at 5), six shapes 5 (4e6 walkers x
-// 1000 steps 75 ms against 88 with the kernel of eight at 4).  RS and ERL keep a
-// step's start beside the state and would spill at 8.
+// the compiler's choice).  The plain form's elastic-collision kernels: 7 (72
+// registers, spills of a few words), whose warps hide the latency of long
+// dependent chains: 3.3e5 walkers x 3000 steps 110.4 ms against 112.5 at 6.  The
+// FP32 form's: as many blocks as their phases leave registers for without spills
+// -- one shape 8 (64 registers: 21.8 ms for 1e6 walkers x 2000 steps on
+// 200x200x400 axons against 22.0 ms at 9 with small spills and 22.5 ms at 7;
+// absorbing membranes, 3e5 walkers x 3000 steps, 14.7 ms against 16.6 at 5), six
+// shapes 5 (4e6 walkers x 1000 steps 75 ms against 88 with the kernel of eight
+// at 4).  RS and ERL keep a step's start beside the state and would spill at 8.
 template <typename Real, int NS, bool HASH, int IM, bool MT>
 constexpr int walk_min_blocks()
 {
-    if (std::is_same<Real, double>::value) return NS == 1 ? 5 : 0;
+    if (std::is_same<Real, double>::value) return HASH || IM != kInteractEC || MT ? 5 : 7;
     if (HASH) return NS == 1 && IM == kInteractEC && !MT ? 7 : 0;  // the verification kernel would spill at 8
     if (IM != kInteractEC) return NS == 1 && IM == kInteractRS && !MT ? 7 : 0;
     return NS == 1 ? 8 : NS == 2 ? (MT ? 7 : 8) : NS == 3 ? 7 : NS == 4 ? 6 : NS == 6 ? 5 : 4;
@@ -929,7 +1016,7 @@ walk_kernel(Geometry g, Tables<Real> t, WalkerState<Real> st, RunCtl ctl, int64_
 // a block of walkers of one request for that request's next steps.  The
 // request descriptors and the task table are read once per block.
 template <typename Real, int NS>
-__global__ void __launch_bounds__(kWalkBlock, std::is_same<Real, double>::value || NS > 4 ? 4 : NS > 2 ? 6 : 8)
+__global__ void __launch_bounds__(kWalkBlock, std::is_same<Real, double>::value ? 5 : NS > 4 ? 4 : NS > 2 ? 6 : 8)
 walk_batched_kernel(const ReqDesc<Real> *reqs, const BlockTask *tasks, int32_t n_tasks)
 {
     if ((int32_t)blockIdx.x >= n_tasks) return;
@@ -949,15 +1036,19 @@ cudaError_t launch_walk_batched(int ns_bucket, int32_t n_tasks, cudaStream_t str
                                 const BlockTask *tasks)
 {
     if (n_tasks <= 0) return cudaSuccess;
-    const dim3 grid((unsigned)n_tasks);
+    const unsigned grid = (unsigned)n_tasks;
+#define RMS_BATCHED(NS)                                                                                             \
+    walk_batched_kernel<Real, NS>                                                                                   \
+        <<<grid, kWalkBlock, Phases<Real, NS>::bytes(NS), stream>>>(reqs, tasks, n_tasks)
     if (ns_bucket <= 1)
-        walk_batched_kernel<Real, 1><<<grid, kWalkBlock, 0, stream>>>(reqs, tasks, n_tasks);
+        RMS_BATCHED(1);
     else if (ns_bucket <= 2)
-        walk_batched_kernel<Real, 2><<<grid, kWalkBlock, 0, stream>>>(reqs, tasks, n_tasks);
+        RMS_BATCHED(2);
     else if (ns_bucket <= 4)
-        walk_batched_kernel<Real, 4><<<grid, kWalkBlock, 0, stream>>>(reqs, tasks, n_tasks);
+        RMS_BATCHED(4);
     else
-        walk_batched_kernel<Real, 8><<<grid, kWalkBlock, 0, stream>>>(reqs, tasks, n_tasks);
+        RMS_BATCHED(8);
+#undef RMS_BATCHED
     return cudaGetLastError();
 }
 
@@ -969,13 +1060,17 @@ int batched_blocks_per_sm(int ns_bucket)
     int n = 0;
     cudaError_t e;
     if (ns_bucket <= 1)
-        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, walk_batched_kernel<Real, 1>, kWalkBlock, 0);
+        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, walk_batched_kernel<Real, 1>, kWalkBlock,
+                                                          (Phases<Real, 1>::bytes(1)));
     else if (ns_bucket <= 2)
-        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, walk_batched_kernel<Real, 2>, kWalkBlock, 0);
+        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, walk_batched_kernel<Real, 2>, kWalkBlock,
+                                                          (Phases<Real, 2>::bytes(2)));
     else if (ns_bucket <= 4)
-        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, walk_batched_kernel<Real, 4>, kWalkBlock, 0);
+        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, walk_batched_kernel<Real, 4>, kWalkBlock,
+                                                          (Phases<Real, 4>::bytes(4)));
     else
-        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, walk_batched_kernel<Real, 8>, kWalkBlock, 0);
+        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, walk_batched_kernel<Real, 8>, kWalkBlock,
+                                                          (Phases<Real, 8>::bytes(8)));
     return e == cudaSuccess && n > 0 ? n : 1;
 }
 
@@ -989,20 +1084,25 @@ cudaError_t launch_walk(int n_shapes, bool hash, dim3 grid, cudaStream_t stream,
                         int64_t k_begin, int64_t k_end, int32_t rec)
 {
 #define RMS_LAUNCH(NSV, HASHV, RELAXV)                                                                     \
-    walk_kernel<Real, NSV, HASHV, IM, MT, RELAXV><<<grid, kWalkBlock, 0, stream>>>(g, t, st, ctl, k_begin, \
+    walk_kernel<Real, NSV, HASHV, IM, MT, RELAXV><<<grid, kWalkBlock, Phases<Real, NSV>::bytes(n_shapes), stream>>>( \
+        g, t, st, ctl, k_begin, \
                                                                                   k_end, rec)
-// kernels of three and six shapes where they pay: the FP32 form's elastic collision
+// the plain form: one shape, or any (its phases are in shared memory); kernels of
+// three and six shapes where they pay: the FP32 form's elastic collision
 #define RMS_LAUNCH_NS(HASHV, RELAXV)                                                  \
     do {                                                                              \
-        constexpr bool kMore = !std::is_same<Real, double>::value && IM == kInteractEC && !MT && !HASHV; \
+        constexpr bool kPlain = std::is_same<Real, double>::value;                    \
+        constexpr bool kMore = !kPlain && IM == kInteractEC && !MT && !HASHV;         \
         if (n_shapes <= 1)                                                            \
             RMS_LAUNCH(1, HASHV, RELAXV);                                             \
+        else if (kPlain)                                                              \
+            RMS_LAUNCH(8, HASHV, RELAXV);                                             \
         else if (n_shapes <= 2)                                                       \
-            RMS_LAUNCH(2, HASHV, RELAXV);                                             \
+            RMS_LAUNCH(kPlain ? 8 : 2, HASHV, RELAXV);                                             \
         else if (kMore && n_shapes <= 3)                                              \
-            RMS_LAUNCH(kMore ? 3 : 4, HASHV, RELAXV);                                 \
+            RMS_LAUNCH(kMore ? 3 : 8, HASHV, RELAXV);                                 \
         else if (n_shapes <= 4)                                                       \
-            RMS_LAUNCH(4, HASHV, RELAXV);                                             \
+            RMS_LAUNCH(kPlain ? 8 : 4, HASHV, RELAXV);                                             \
         else if (kMore && n_shapes <= 6)                                              \
             RMS_LAUNCH(kMore ? 6 : 8, HASHV, RELAXV);                                 \
         else                                                                          \

@@ -15,7 +15,9 @@
 // order: the same bits.
 //
 // 600 steps of 1e4 walkers on 64^3 axons: 2.39 ms against 4.50 (one warp on each
-// of 313 schedulers before; now two on each).
+// of 313 schedulers before; now two on each).  Seven blocks an SM (72 registers)
+// rather than five: no difference up to 24 000 walkers, 4.08 ms against 4.53 for
+// 30 000.
 #pragma once
 
 #include "walk_kernel.cuh"
@@ -25,7 +27,7 @@ namespace rms {
 constexpr int kQuadWalkers = 32;  // walkers of a block of kWalkBlock threads: a warp of the one-thread kernel
 
 template <int NS, int RELAX>
-__global__ void __launch_bounds__(kWalkBlock, NS == 1 ? 5 : 0)
+__global__ void __launch_bounds__(kWalkBlock, NS == 1 ? 7 : 0)
 walk_quad_kernel(Geometry g, Tables<double> t, WalkerState<double> st, RunCtl ctl, int64_t k_begin, int64_t k_end,
                  int32_t rec)
 {
@@ -85,7 +87,7 @@ walk_quad_kernel(Geometry g, Tables<double> t, WalkerState<double> st, RunCtl ct
             const U4 x = philox4x32_10_rk(
                 U4{(uint32_t)w, (uint32_t)(w >> 32), (uint32_t)(k + ax), kTagDir << 16}, rk);
             double n3[3];
-            direction_from(x.x, x.y, t.trig, n3);
+            direction_from<true>(x.x, x.y, t.trig, n3);
             __syncwarp();
             s_n[threadIdx.x][0] = n3[0];
             s_n[threadIdx.x][1] = n3[1];
