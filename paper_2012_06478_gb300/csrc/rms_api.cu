@@ -233,8 +233,9 @@ __global__ void trig_table_kernel(double *trig)
 
 // Per step: the weights dt G_{s,k} (rows of `pitch`, zeros beyond the last
 // step) and the step flags.
+// Sets bit 1 of warn where a weight is out of the unchecked arithmetic's range.
 __global__ void step_tables_kernel(int64_t N, int64_t pitch, int32_t S, double dt, const double *G, double *wG64,
-                                   float *wG32, uint8_t *flags)
+                                   float *wG32, uint8_t *flags, int32_t *warn)
 {
     const int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;  // 0-based step index
     if (k >= pitch) return;
@@ -244,6 +245,7 @@ __global__ void step_tables_kernel(int64_t N, int64_t pitch, int32_t S, double d
         wG64[(int64_t)s * pitch + k] = w;
         wG32[(int64_t)s * pitch + k] = (float)w;
         if (w != 0.0) f = 1u;
+        if (!(w == 0.0 || (fabs(w) >= 0x1p-400 && fabs(w) <= 0x1p400))) atomicOr(warn, 2);
     }
     flags[k] = f;
 }
@@ -743,6 +745,21 @@ static void free_sequence(rms_sequence *q, cudaStream_t st)
         if (x) cudaFreeAsync(x, st);
 }
 
+// Whether a step's numbers stay where the plain form's arithmetic needs no range
+// checks (walk_kernel.cuh, SANE): step lengths, voxel and relaxation rates; the
+// weights are looked at on the device, a resumed state when it comes.
+static bool sane_ranges(const rms_substrate *sub, double dt)
+{
+    if (!(sub->voxel_um >= 0x1p-200 && sub->voxel_um <= 0x1p200)) return false;
+    for (int c = 0; c < sub->L; ++c) {
+        const double s = std::sqrt((6.0 * sub->D[c]) * dt) / sub->voxel_um;
+        if (!(s >= 0x1p-200 && s <= 0x1p200)) return false;
+        for (const double T : {sub->T2[c], sub->T1[c]})
+            if (!std::isinf(T) && !(dt / T >= 0x1p-400 && dt / T <= 0x1p400)) return false;
+    }
+    return true;
+}
+
 static rms_status set_sequence_impl(rms_substrate *sub, const rms_sequence_desc *d, rms_sequence *q,
                                     bool *warn)
 {
@@ -817,7 +834,7 @@ static rms_status set_sequence_impl(rms_substrate *sub, const rms_sequence_desc 
         RMS_CUDA(cudaMemcpyAsync(q->d_T, hostT.data(), sizeof(uint32_t) * hostT.size(), cudaMemcpyHostToDevice, st));
     }
     step_tables_kernel<<<(unsigned)((q->pitch + 255) / 256), 256, 0, st>>>(N, q->pitch, S, d->dt_ms, d_G, q->d_wG64,
-                                                                            q->d_wG32, q->d_flags);
+                                                                            q->d_wG32, q->d_flags, d_warn);
     bvalue_kernel<<<(unsigned)std::max(S, 1), kBvThreads, 0, st>>>(N, S, d->dt_ms, d_G, d->n_b, q->d_b, q->d_bs,
                                                                     q->d_q);
     RMS_CUDA(cudaGetLastError());
@@ -826,7 +843,8 @@ static rms_status set_sequence_impl(rms_substrate *sub, const rms_sequence_desc 
     RMS_CUDA(cudaFreeAsync(d_G, st));
     RMS_CUDA(cudaFreeAsync(d_warn, st));
     RMS_CUDA(cudaStreamSynchronize(st));
-    *warn = w != 0 || host_warn;
+    *warn = (w & 1) != 0 || host_warn;
+    q->sane = (w & 2) == 0 && sane_ranges(sub, d->dt_ms);
     return RMS_OK;
 }
 
@@ -937,6 +955,7 @@ ReqDesc<Real> rms::run_desc(rms_run_handle *r)
     d.ctl.cancel = r->d_cancel;
     d.ctl.mom_partial = r->d_mom_partial;
     d.ctl.n_blocks = r->n_blocks;
+    d.ctl.sane = q->sane && r->sane;
     round_keys(r->seed, d.ctl.rk);
     return d;
 }
@@ -1137,11 +1156,11 @@ rms_status rms::run_setup(rms_run_handle *r, bool with_cancel_and_events)
 // writes).  The FP32 form splits each double into its float and the Kahan
 // compensation (float - double), so the compensated value is the double's
 // to within float rounding of the difference; a saturated walker (+inf)
-// keeps kSaturatedF.
+// keeps kSaturatedF.  Sets odd where an offset is not +0 or in [2^-300, 1].
 template <typename Real>
 __global__ void import_kernel(WalkerState<Real> st, int64_t W, int32_t S, const int32_t *i, const double *o,
                               const int32_t *i0, const double *o0, const int32_t *c, const double *A,
-                              const double *phase, const uint64_t *hash)
+                              const double *phase, const uint64_t *hash, int32_t *odd)
 {
     const int64_t w = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (w >= W) return;
@@ -1149,6 +1168,8 @@ __global__ void import_kernel(WalkerState<Real> st, int64_t W, int32_t S, const 
     for (int a = 0; a < 3; ++a) {
         st.o[a][w] = (Real)o[3 * w + a];
         st.o0[a][w] = (Real)o0[3 * w + a];
+        for (const double x : {o[3 * w + a], o0[3 * w + a]})
+            if (!(__double_as_longlong(x) == 0 || (x >= 0x1p-300 && x <= 1.0))) *odd = 1;
         st.i0[a][w] = i0[3 * w + a];
         st.di[a][w] = i[3 * w + a] - i0[3 * w + a];
     }
@@ -1205,20 +1226,24 @@ static rms_status run_import(rms_run_handle *r, const rms_run_state *from)
     RMS_TRY(upload(&d_ph, from->phase, (size_t)3 * S * W, s));
     if (from->hash) RMS_TRY(upload(&d_h, from->hash, (size_t)W, s));
     const unsigned nb = (unsigned)((W + 255) / 256);
+    int32_t *d_odd = nullptr, odd = 0;
+    RMS_TRY(upload(&d_odd, &odd, 1, s));
     if (r->precision == RMS_FP32)
-        import_kernel<float><<<nb, 256, 0, s>>>(r->st32, W, S, d_i, d_o, d_i0, d_o0, d_c, d_A, d_ph, d_h);
+        import_kernel<float><<<nb, 256, 0, s>>>(r->st32, W, S, d_i, d_o, d_i0, d_o0, d_c, d_A, d_ph, d_h, d_odd);
     else
-        import_kernel<double><<<nb, 256, 0, s>>>(r->st64, W, S, d_i, d_o, d_i0, d_o0, d_c, d_A, d_ph, d_h);
+        import_kernel<double><<<nb, 256, 0, s>>>(r->st64, W, S, d_i, d_o, d_i0, d_o0, d_c, d_A, d_ph, d_h, d_odd);
     RMS_CUDA(cudaGetLastError());
+    RMS_CUDA(cudaMemcpyAsync(&odd, d_odd, sizeof odd, cudaMemcpyDeviceToHost, s));
     if (from->moments)
         for (int rr = 0; rr < q->n_rec; ++rr)
             if (q->rec_steps[rr] <= from->step)
                 RMS_CUDA(cudaMemcpyAsync(r->d_mom_partial + (size_t)rr * r->n_blocks * mom_sub(r) * kMoments,
                                          from->moments + 22 * rr, sizeof(double) * kMoments, cudaMemcpyHostToDevice, s));
-    void *tmp[] = {d_i, d_i0, d_c, d_o, d_o0, d_A, d_ph, d_h};
+    void *tmp[] = {d_i, d_i0, d_c, d_o, d_o0, d_A, d_ph, d_h, d_odd};
     for (void *x : tmp)
         if (x) RMS_CUDA(cudaFreeAsync(x, s));
     RMS_CUDA(cudaStreamSynchronize(s));  // the host arrays may go once this returns
+    r->sane = odd == 0;
     return RMS_OK;
 }
 

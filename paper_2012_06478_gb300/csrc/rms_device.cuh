@@ -204,6 +204,7 @@ struct RunCtl {
     const volatile int32_t *cancel; // host-mapped cancel flag (nullptr = none)
     double *mom_partial;            // [rec][block][22]
     int32_t n_blocks;
+    int32_t sane;                   // numbers in the ranges of unchecked arithmetic (plain form)
     uint32_t rk[kRoundKeys];        // Philox round keys of seed (round_keys)
 };
 

@@ -52,6 +52,7 @@ struct rms_sequence {
     int32_t S = 0, n_dirs = 0, n_b = 0, n_rec = 0;
     int32_t any_relax = 0;
     int32_t has_mode = 0;
+    bool sane = false;  // numbers in the ranges of unchecked arithmetic (walk_kernel.cuh)
     std::vector<int64_t> rec_steps;  // host copy of the recording steps
     double *d_s64 = nullptr, *d_dtR64 = nullptr, *d_wG64 = nullptr;
     float *d_s32 = nullptr, *d_dtR32 = nullptr, *d_wG32 = nullptr;
@@ -72,6 +73,7 @@ struct rms_run_handle {
     int32_t precision = RMS_FP64;
     uint32_t flags = 0;
     int32_t interaction = RMS_EC;
+    bool sane = true;  // and the state's offsets
     cudaStream_t stream = nullptr;
     int32_t n_blocks = 0;
     bool quad = false;  // four lanes to a walker (walk_quad.cuh); moment partials per 32 walkers

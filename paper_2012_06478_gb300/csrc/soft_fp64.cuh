@@ -110,22 +110,15 @@ __host__ __device__ __forceinline__ int64_t smulhi(uint64_t x, int64_t e)
     return e < 0 ? -(int64_t)m : (int64_t)m;
 }
 
-// a / b for a >= +0 and b > +0 (sign bits clear).  Returns false when a or b
-// is subnormal, infinite or NaN, or the quotient leaves the normal range
-// (except an overflow to infinity by rounding, which is the IEEE result).
-__host__ __device__ __forceinline__ bool div_pos(double a, double b, double &q)
+// a / b for a and b known to be normal and positive, with a quotient known to be
+// normal (the caller's ranges guarantee it).
+__host__ __device__ __forceinline__ double div_normal(double a, double b)
 {
     const uint64_t ua = bits_of(a), ub = bits_of(b);
-    if (ua == 0) {  // 0 / b = +0
-        q = 0.0;
-        return true;
-    }
     const int32_t ea = (int32_t)(ua >> 52), eb = (int32_t)(ub >> 52);
-    if ((uint32_t)(ea - 1) >= 0x7FEu || (uint32_t)(eb - 1) >= 0x7FEu) return false;
     const uint64_t A = (ua & kMant) | kHidden, B = (ub & kMant) | kHidden;  // [2^52, 2^53)
     const bool ge = A >= B;
     const int32_t e = ea - eb + 1022 + (ge ? 1 : 0);  // biased exponent of the quotient
-    if ((uint32_t)(e - 1) >= 0x7FEu) return false;
     // x ~ 2^115 / B in (2^62, 2^63]: seed from the single-precision reciprocal
     // of B's top 24 bits (relative error below 2^-22), exact as a shifted
     // integer; then two Newton steps x += x e / 2^115, e = 2^115 - B x
@@ -156,7 +149,24 @@ __host__ __device__ __forceinline__ bool div_pos(double a, double b, double &q)
     // round to nearest, ties to even (no ties occur for a quotient): up iff
     // 2R > B, or 2R == B and Q odd
     const uint64_t up = ((uint64_t)R << 1) + (Q & 1ULL) > B ? 1ULL : 0ULL;
-    q = double_of((((uint64_t)(e - 1)) << 52) + Q + up);  // Q carries the hidden bit; a carry moves into the exponent
+    return double_of((((uint64_t)(e - 1)) << 52) + Q + up);  // Q carries the hidden bit; a carry moves into the exponent
+}
+
+// a / b for a >= +0 and b > +0 (sign bits clear).  Returns false when a or b
+// is subnormal, infinite or NaN, or the quotient leaves the normal range
+// (except an overflow to infinity by rounding, which is the IEEE result).
+__host__ __device__ __forceinline__ bool div_pos(double a, double b, double &q)
+{
+    const uint64_t ua = bits_of(a), ub = bits_of(b);
+    if (ua == 0) {  // 0 / b = +0
+        q = 0.0;
+        return true;
+    }
+    const int32_t ea = (int32_t)(ua >> 52), eb = (int32_t)(ub >> 52);
+    if ((uint32_t)(ea - 1) >= 0x7FEu || (uint32_t)(eb - 1) >= 0x7FEu) return false;
+    const int32_t e = ea - eb + 1022 + ((ua & kMant) >= (ub & kMant) ? 1 : 0);
+    if ((uint32_t)(e - 1) >= 0x7FEu) return false;
+    q = div_normal(a, b);
     return true;
 }
 

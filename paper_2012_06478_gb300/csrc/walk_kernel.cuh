@@ -102,7 +102,6 @@ static __device__ __noinline__ double hw_div(double a, double b) { return a / b;
 
 // FP64 products and quotients of non-negative operands on the integer ALU
 // (sfp::mul_rn, div_pos: the IEEE results bit for bit).
-// mulr is the product of the form: this one for FP64, a plain multiply for FP32.
 __device__ __forceinline__ double dmul(double a, double b)
 {
     double p;
@@ -116,8 +115,69 @@ __device__ __forceinline__ double ddiv_nn(double a, double b)
     return q;
 }
 
-__device__ __forceinline__ double mulr(double a, double b) { return dmul(a, b); }
-__device__ __forceinline__ float mulr(float a, float b) { return a * b; }
+// SANE: the run's numbers are within ranges (sane_ranges, rms_api.cu) where every
+// operand and result of the step is zero or far inside the normal numbers: no
+// range checks, no branches to the hardware operations -- a fifth of the step's
+// instructions.  Otherwise the checked versions.  The same bits.
+//
+// Why the ranges hold: steps are 2^-200 to 1 voxels and directions' components at
+// least 2^-60; offsets are 0 or, but for a chance of 2^-300, above 2^-300; so face
+// times, their differences and all products stay above 2^-900, and quotients
+// below 2^300.
+__device__ __forceinline__ bool is_zero(double x)  // of a zero or normal number
+{
+    return (__double2hiint(x) & 0x7FF00000) == 0;
+}
+// the product where neither operand is zero (SANE)
+template <bool SANE>
+__device__ __forceinline__ double times_nz(double a, double b)
+{
+    if constexpr (SANE)
+        return sfp::mul_normal(a, b);
+    else
+        return dmul(a, b);
+}
+// where a may be
+template <bool SANE>
+__device__ __forceinline__ double times(double a, double b)
+{
+    if constexpr (SANE) {
+        const double p = sfp::mul_normal(a, b);
+        return is_zero(a) ? __hiloint2double((__double2hiint(a) ^ __double2hiint(b)) & (int)0x80000000, 0) : p;
+    } else {
+        return dmul(a, b);
+    }
+}
+// where both may be
+template <bool SANE>
+__device__ __forceinline__ double times_any(double a, double b)
+{
+    if constexpr (SANE) {
+        const double p = sfp::mul_normal(a, b);
+        return is_zero(a) || is_zero(b)
+                   ? __hiloint2double((__double2hiint(a) ^ __double2hiint(b)) & (int)0x80000000, 0)
+                   : p;
+    } else {
+        return dmul(a, b);
+    }
+}
+// a / b for a >= +0, b > 0
+template <bool SANE>
+__device__ __forceinline__ double over(double a, double b)
+{
+    if constexpr (SANE) {
+        const double q = sfp::div_normal(a, b);
+        return is_zero(a) ? 0.0 : q;
+    } else {
+        return ddiv_nn(a, b);
+    }
+}
+
+template <bool SANE = false>
+__device__ __forceinline__ float times_any(float a, float b)
+{
+    return a * b;
+}
 
 // Exact doubles built from their bits on the integer ALU, so that values
 // which need no rounding do not occupy GB300's narrow FP64 pipe.
@@ -353,16 +413,16 @@ struct Phases {
         for (int k = 0; k < 3 * n; ++k) st.phase[k * W + li] = p[k * kWalkBlock];
     }
     // component `axis` of every shape's phase += w dx
-    template <typename Weight>
+    template <bool SANE, typename Weight>
     __device__ __forceinline__ void add(int n, int axis, double dx, Weight weight)
     {
         if constexpr (NS == 1) {
-            p[axis * kWalkBlock] = p[axis * kWalkBlock] + dmul(weight(0), dx);
+            p[axis * kWalkBlock] = p[axis * kWalkBlock] + times_any<SANE>(weight(0), dx);
         } else {
 #pragma unroll 1
             for (int s = 0; s < n; ++s) {
                 double &x = p[(3 * s + axis) * kWalkBlock];
-                x = x + dmul(weight(s), dx);
+                x = x + times_any<SANE>(weight(s), dx);
             }
         }
     }
@@ -488,7 +548,7 @@ __device__ __forceinline__ void warp_moments(double al, const double dx[3], doub
 // otherwise read them at every draw (the batched kernel, whose request
 // descriptors sit in shared memory).  `rec` is the first recording step's
 // index beyond k_begin.
-template <typename Real, int NS, bool HASH, int IM, bool MT, int RELAX, bool RK = false>
+template <typename Real, int NS, bool HASH, int IM, bool MT, int RELAX, bool RK = false, bool SANE = false>
 __device__ __forceinline__ void walk_block(const Geometry &g, const Tables<Real> &t, const WalkerState<Real> &st,
                                            const RunCtl &ctl, int64_t block, int64_t k_begin, int64_t k_end,
                                            int32_t rec)
@@ -684,12 +744,12 @@ __device__ __forceinline__ void walk_block(const Geometry &g, const Tables<Real>
                 // outside its range, e.g. o = -0)
                 double T[3] = {};
                 const auto face_time = [](double o, double d) {
-                    return ddiv_nn(dgt0(d) ? 1.0 - o : o, __longlong_as_double(dbits(d) & 0x7FFFFFFFFFFFFFFFLL));
+                    return over<SANE>(dgt0(d) ? 1.0 - o : o, __longlong_as_double(dbits(d) & 0x7FFFFFFFFFFFFFFFLL));
                 };
 #pragma unroll 1
                 for (int r = 0; r < 3; ++r) {
-                    d[0] = dmul(n[0], sc);
-                    T[0] = (dgt0(d[0]) || dlt0(d[0])) ? face_time(o[0], d[0]) : kInf;
+                    d[0] = times_nz<SANE>(n[0], sc);
+                    T[0] = SANE || dgt0(d[0]) || dlt0(d[0]) ? face_time(o[0], d[0]) : kInf;
                     rotate(n);
                     rotate(o);
                     rotate(d);
@@ -714,7 +774,7 @@ __device__ __forceinline__ void walk_block(const Geometry &g, const Tables<Real>
                     }
                     if (!dlt_nn(tmin, 1.0)) break;
                     const double dts = tmin - tau;
-                    if (relax) A = A + dmul(dts, rate);
+                    if (relax) A = A + times_any<SANE>(dts, rate);
                     tau = tmin;
                     if constexpr (HASH) ++nev;
                     const bool up = dgt0(best == 2 ? d[2] : (best == 1 ? d[1] : d[0]));
@@ -725,7 +785,7 @@ __device__ __forceinline__ void walk_block(const Geometry &g, const Tables<Real>
                         double da = best == 0 ? d[1] : d[0], db = best == 2 ? d[1] : d[2];
 #pragma unroll 1
                         for (int r = 0; r < 2; ++r) {
-                            const double x = dclamp01(oa + dmul(dts, da)), y = da;
+                            const double x = dclamp01(oa + times<SANE>(dts, da)), y = da;
                             oa = ob;
                             ob = x;
                             da = db;
@@ -762,7 +822,7 @@ __device__ __forceinline__ void walk_block(const Geometry &g, const Tables<Real>
                                 sc = sn;
 #pragma unroll 1
                                 for (int r = 0; r < 3; ++r) {
-                                    d[0] = dmul(n[0], sc);
+                                    d[0] = times_nz<SANE>(n[0], sc);
                                     if (dbits(T[0]) != 0x7FF0000000000000LL) T[0] = tau + face_time(o[0], d[0]);
                                     rotate(n);
                                     rotate(o);
@@ -782,11 +842,11 @@ __device__ __forceinline__ void walk_block(const Geometry &g, const Tables<Real>
                     const double rem = 1.0 - tau;
 #pragma unroll 1
                     for (int r = 0; r < 3; ++r) {
-                        o[0] = dclamp01(o[0] + dmul(rem, d[0]));
+                        o[0] = dclamp01(o[0] + times_nz<SANE>(rem, d[0]));
                         rotate(o);
                         rotate(d);
                     }
-                    if (relax) A = A + dmul(rem, rate);
+                    if (relax) A = A + times_any<SANE>(rem, rate);
                 }
             } else {
                 // Precision form: the same walk in FP32.  The choices are selects and
@@ -924,7 +984,8 @@ __device__ __forceinline__ void walk_block(const Geometry &g, const Tables<Real>
             if constexpr (kF64) {
 #pragma unroll 1
                 for (int r = 0; r < 3; ++r) {
-                    ph.add(ctl.n_shapes, r, dmul(lp, (double)di[0] + (o[0] - ph.start[r * kWalkBlock])), weight);
+                    ph.template add<SANE>(ctl.n_shapes, r,
+                                          times<SANE>((double)di[0] + (o[0] - ph.start[r * kWalkBlock]), lp), weight);
                     rotate(o);
                     rotate(di);
                 }
@@ -1005,11 +1066,11 @@ constexpr int walk_min_blocks()
 }
 
 // One run: block b of the grid advances walkers b*kWalkBlock ... of the run.
-template <typename Real, int NS, bool HASH, int IM, bool MT, int RELAX>
+template <typename Real, int NS, bool HASH, int IM, bool MT, int RELAX, bool SANE>
 __global__ void __launch_bounds__(kWalkBlock, (walk_min_blocks<Real, NS, HASH, IM, MT>()))
 walk_kernel(Geometry g, Tables<Real> t, WalkerState<Real> st, RunCtl ctl, int64_t k_begin, int64_t k_end, int32_t rec)
 {
-    walk_block<Real, NS, HASH, IM, MT, RELAX, true>(g, t, st, ctl, blockIdx.x, k_begin, k_end, rec);
+    walk_block<Real, NS, HASH, IM, MT, RELAX, true, SANE>(g, t, st, ctl, blockIdx.x, k_begin, k_end, rec);
 }
 
 // Many runs in one launch (continuous batching): block i executes task i --
@@ -1083,10 +1144,19 @@ cudaError_t launch_walk(int n_shapes, bool hash, dim3 grid, cudaStream_t stream,
                         const Tables<Real> &t, const WalkerState<Real> &st, const RunCtl &ctl,
                         int64_t k_begin, int64_t k_end, int32_t rec)
 {
-#define RMS_LAUNCH(NSV, HASHV, RELAXV)                                                                     \
-    walk_kernel<Real, NSV, HASHV, IM, MT, RELAXV><<<grid, kWalkBlock, Phases<Real, NSV>::bytes(n_shapes), stream>>>( \
-        g, t, st, ctl, k_begin, \
-                                                                                  k_end, rec)
+    // the checked products and quotients: the verification kernel, the other
+    // interactions and absorbing membranes, and numbers out of range
+    constexpr bool kSane = std::is_same<Real, double>::value && IM == kInteractEC && !MT;
+#define RMS_LAUNCH_AS(NSV, HASHV, RELAXV, SANEV)                                                                \
+    walk_kernel<Real, NSV, HASHV, IM, MT, RELAXV, SANEV>                                                        \
+        <<<grid, kWalkBlock, Phases<Real, NSV>::bytes(n_shapes), stream>>>(g, t, st, ctl, k_begin, k_end, rec)
+#define RMS_LAUNCH(NSV, HASHV, RELAXV)                                  \
+    do {                                                                \
+        if (kSane && !HASHV && ctl.sane)                                \
+            RMS_LAUNCH_AS(NSV, HASHV, RELAXV, (kSane && !HASHV));       \
+        else                                                            \
+            RMS_LAUNCH_AS(NSV, HASHV, RELAXV, false);                   \
+    } while (0)
 // the plain form: one shape, or any (its phases are in shared memory); kernels of
 // three and six shapes where they pay: the FP32 form's elastic collision
 #define RMS_LAUNCH_NS(HASHV, RELAXV)                                                  \
@@ -1118,6 +1188,7 @@ cudaError_t launch_walk(int n_shapes, bool hash, dim3 grid, cudaStream_t stream,
         RMS_LAUNCH_NS(false, 0);
 #undef RMS_LAUNCH_NS
 #undef RMS_LAUNCH
+#undef RMS_LAUNCH_AS
     return cudaGetLastError();
 }
 

@@ -26,7 +26,7 @@ namespace rms {
 
 constexpr int kQuadWalkers = 32;  // walkers of a block of kWalkBlock threads: a warp of the one-thread kernel
 
-template <int NS, int RELAX>
+template <int NS, int RELAX, bool SANE>
 __global__ void __launch_bounds__(kWalkBlock, NS == 1 ? 7 : 0)
 walk_quad_kernel(Geometry g, Tables<double> t, WalkerState<double> st, RunCtl ctl, int64_t k_begin, int64_t k_end,
                  int32_t rec)
@@ -99,10 +99,10 @@ walk_quad_kernel(Geometry g, Tables<double> t, WalkerState<double> st, RunCtl ct
         double n = from[a];
         double rate = kZero;
         if (relax) rate = __ldg(t.dtR + mode * L + c);
-        double d = dmul(n, sc);
+        double d = times_nz<SANE>(n, sc);
         double T = kInf;
-        if (ax < 3 && (dgt0(d) || dlt0(d)))
-            T = ddiv_nn(dgt0(d) ? 1.0 - o : o, __longlong_as_double(dbits(d) & 0x7FFFFFFFFFFFFFFFLL));
+        if (ax < 3 && (SANE || dgt0(d) || dlt0(d)))
+            T = over<SANE>(dgt0(d) ? 1.0 - o : o, __longlong_as_double(dbits(d) & 0x7FFFFFFFFFFFFFFFLL));
         double tau = kZero;
 #pragma unroll 1
         for (int ev = 0; ev < 3; ++ev) {
@@ -123,14 +123,14 @@ walk_quad_kernel(Geometry g, Tables<double> t, WalkerState<double> st, RunCtl ct
                 const int best = __ffs((int)(at & 7u)) - 1;
                 const bool up = ((ups >> best) & 1u) != 0u, mine = ax == best;
                 const double dts = tmin - tau;
-                if (relax) A = A + dmul(dts, rate);
+                if (relax) A = A + times_any<SANE>(dts, rate);
                 tau = tmin;
                 if (mine) {
                     T = kInf;
                     o = up ? 0.0 : 1.0;
                     di += up ? 1 : -1;
                 } else {
-                    o = dclamp01(o + dmul(dts, d));
+                    o = dclamp01(o + times<SANE>(dts, d));
                 }
                 const int32_t sb = best == 2 ? sz : (best == 1 ? sy : 1);
                 const uint32_t bit = (best == 2 ? kFaceZ : (best == 1 ? kFaceY : kFaceX)) << (up ? 3 : 0);
@@ -154,9 +154,9 @@ walk_quad_kernel(Geometry g, Tables<double> t, WalkerState<double> st, RunCtl ct
                             const double sn = __ldg(t.s + c);
                             if (dbits(sn) != dbits(sc)) {
                                 sc = sn;
-                                d = dmul(n, sc);
+                                d = times_nz<SANE>(n, sc);
                                 if (dbits(T) != 0x7FF0000000000000LL)
-                                    T = tau + ddiv_nn(dgt0(d) ? 1.0 - o : o,
+                                    T = tau + over<SANE>(dgt0(d) ? 1.0 - o : o,
                                                       __longlong_as_double(dbits(d) & 0x7FFFFFFFFFFFFFFFLL));
                             }
                         } else {  // reflected: stays in its voxel, at the face
@@ -175,15 +175,15 @@ walk_quad_kernel(Geometry g, Tables<double> t, WalkerState<double> st, RunCtl ct
             }
         }
         const double rem = 1.0 - tau;
-        o = dclamp01(o + dmul(rem, d));
-        if (relax) A = A + dmul(rem, rate);
+        o = dclamp01(o + times_nz<SANE>(rem, d));
+        if (relax) A = A + times_any<SANE>(rem, rate);
         // ---- phase (Eq. 7)
         if (graded) {
-            const double dx = dmul(lp, (double)di + (o - o0));
+            const double dx = times<SANE>((double)di + (o - o0), lp);
 #pragma unroll
             for (int s = 0; s < NS; ++s)
                 if (s < ctl.n_shapes)
-                    ph[s] = ph[s] + dmul(NS == 1 ? wg : __ldg(t.wG + (int64_t)s * t.pitch + (k - 1)), dx);
+                    ph[s] = ph[s] + times_any<SANE>(NS == 1 ? wg : __ldg(t.wG + (int64_t)s * t.pitch + (k - 1)), dx);
         }
         // ---- displacement moments: the first warp sums the block's 32 walkers as
         //      the one-thread kernel's warp does

@@ -10,12 +10,18 @@ cudaError_t launch_walk_quad(int n_shapes, cudaStream_t stream, const Geometry &
                              int32_t rec)
 {
     const unsigned grid = (unsigned)((ctl.n_walkers + kQuadWalkers - 1) / kQuadWalkers);
-#define RMS_QUAD(NS)                                                                                        \
-    do {                                                                                                    \
-        if (t.any_relax)                                                                                    \
-            walk_quad_kernel<NS, 1><<<grid, kWalkBlock, 0, stream>>>(g, t, st, ctl, k_begin, k_end, rec);   \
-        else                                                                                                \
-            walk_quad_kernel<NS, 0><<<grid, kWalkBlock, 0, stream>>>(g, t, st, ctl, k_begin, k_end, rec);   \
+#define RMS_QUAD_AS(NS, RELAX, SANE) \
+    walk_quad_kernel<NS, RELAX, SANE><<<grid, kWalkBlock, 0, stream>>>(g, t, st, ctl, k_begin, k_end, rec)
+#define RMS_QUAD(NS)                       \
+    do {                                   \
+        if (t.any_relax && ctl.sane)       \
+            RMS_QUAD_AS(NS, 1, true);      \
+        else if (t.any_relax)              \
+            RMS_QUAD_AS(NS, 1, false);     \
+        else if (ctl.sane)                 \
+            RMS_QUAD_AS(NS, 0, true);      \
+        else                               \
+            RMS_QUAD_AS(NS, 0, false);     \
     } while (0)
     if (n_shapes <= 1)
         RMS_QUAD(1);
@@ -26,6 +32,7 @@ cudaError_t launch_walk_quad(int n_shapes, cudaStream_t stream, const Geometry &
     else
         RMS_QUAD(8);
 #undef RMS_QUAD
+#undef RMS_QUAD_AS
     return cudaGetLastError();
 }
 
