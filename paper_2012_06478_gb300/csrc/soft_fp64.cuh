@@ -178,6 +178,25 @@ __host__ __device__ __forceinline__ bool div_pos(double a, double b, double &q)
 __host__ __device__ __forceinline__ double mul_core(uint64_t ua, uint64_t ub, uint64_t lo, uint64_t hi, bool top,
                                                     int32_t e)
 {
+#ifdef __CUDA_ARCH__
+    // The kept bits and, left-aligned, the ones below them by funnel shifts; the
+    // carry of the latter plus one half -- less one unit where the kept part is
+    // even -- is the rounding (10 operations of the ALU in place of 17).
+    const uint32_t s = top ? 11u : 12u;
+    const uint32_t l0 = (uint32_t)lo, l1 = (uint32_t)(lo >> 32), h0 = (uint32_t)hi, h1 = (uint32_t)(hi >> 32);
+    const uint32_t m0 = __funnelshift_l(l1, h0, s), m1 = __funnelshift_l(h0, h1, s);
+    const uint32_t r0 = l0 << s, r1 = __funnelshift_l(l0, l1, s), odd = m0 & 1u;
+    const uint32_t head = ((uint32_t)((ua ^ ub) >> 32) & 0x80000000u) | ((uint32_t)(e - 1) << 20);
+    uint32_t p0, p1;
+    asm("{\n\t.reg .u32 t;\n\t"
+        "add.cc.u32 t, %2, %3;\n\t"
+        "addc.cc.u32 t, %4, %5;\n\t"
+        "addc.cc.u32 %0, %6, 0;\n\t"
+        "addc.u32 %1, %7, %8;\n\t}"
+        : "=r"(p0), "=r"(p1)
+        : "r"(r0), "r"(odd - 1u), "r"(r1), "r"(odd + 0x7FFFFFFFu), "r"(m0), "r"(m1), "r"(head));
+    return __hiloint2double((int)p1, (int)p0);
+#else
     const uint64_t hn = top ? hi : (hi << 1) | (lo >> 63);
     const uint64_t ln = top ? lo : lo << 1;
     const uint64_t M = (hn << 11) | (ln >> 53);  // in [2^52, 2^53)
@@ -185,6 +204,7 @@ __host__ __device__ __forceinline__ double mul_core(uint64_t ua, uint64_t ub, ui
     // up iff rem > 2^52, or rem == 2^52 and M odd
     const uint64_t up = rem + (M & 1ULL) > 0x0010000000000000ULL ? 1ULL : 0ULL;
     return double_of(((ua ^ ub) & 0x8000000000000000ULL) | ((((uint64_t)(e - 1)) << 52) + M + up));
+#endif
 }
 
 // a * b, both finite, normal and of any sign, with a normal product
