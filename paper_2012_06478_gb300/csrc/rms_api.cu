@@ -743,6 +743,7 @@ static void free_sequence(rms_sequence *q, cudaStream_t st)
                  q->d_flags, q->d_mode, q->d_rec_step, q->d_dirs, q->d_b, q->d_bs, q->d_q, q->d_trig};
     for (void *x : p)
         if (x) cudaFreeAsync(x, st);
+    if (q->h_flags) cudaFreeHost(q->h_flags);
 }
 
 // Whether a step's numbers stay where the plain form's arithmetic needs no range
@@ -1072,7 +1073,14 @@ void rms::run_free(rms_run_handle *r, bool sync)
     for (void *x : p)
         if (x) cudaFreeAsync(x, s);
     if (sync || r->h_cancel) cudaStreamSynchronize(s);
-    if (r->h_cancel) cudaFreeHost(r->h_cancel);
+    if (r->h_cancel) {  // no kernel reads it any more
+        if (r->cancel_slot < 0) {
+            cudaFreeHost(r->h_cancel);
+        } else {
+            std::lock_guard<std::mutex> lock(r->seq->flag_mu);
+            r->seq->flags_used &= ~(1ull << r->cancel_slot);
+        }
+    }
     if (r->ev_start) cudaEventDestroy(r->ev_start);
     if (r->ev_end) cudaEventDestroy(r->ev_end);
 }
@@ -1101,6 +1109,29 @@ size_t rms::run_state_bytes(const rms_sequence *q, int64_t W, int32_t precision,
                            (size_t)std::max(q->n_rec, 1) * mom_chunks((int32_t)nb) * kMoments +
                            2 * (size_t)(ncombo + 1) * nc + 4 * (size_t)(ncombo + 1));
     return b;
+}
+
+// A cancel flag for a run: one of its sequence's, or its own.
+static rms_status take_cancel_flag(rms_run_handle *r)
+{
+    rms_sequence *q = r->seq;
+    {
+        std::lock_guard<std::mutex> lock(q->flag_mu);
+        if (!q->h_flags) {
+            int32_t *p = nullptr;
+            RMS_CUDA(cudaHostAlloc((void **)&p, sizeof(int32_t) * rms_sequence::kCancelFlags, cudaHostAllocMapped));
+            q->h_flags = p;
+        }
+        for (int k = 0; k < rms_sequence::kCancelFlags; ++k)
+            if (!((q->flags_used >> k) & 1u)) {
+                q->flags_used |= 1ull << k;
+                r->cancel_slot = k;
+                r->h_cancel = q->h_flags + k;
+                return RMS_OK;
+            }
+    }
+    RMS_CUDA(cudaHostAlloc((void **)&r->h_cancel, sizeof(int32_t), cudaHostAllocMapped));
+    return RMS_OK;
 }
 
 // Allocate the run's device memory (stream-ordered) and lay out the state.
@@ -1143,7 +1174,7 @@ rms_status rms::run_setup(rms_run_handle *r, bool with_cancel_and_events)
     RMS_CUDA(cudaMallocAsync((void **)&r->d_status, sizeof(int32_t), s));
     RMS_CUDA(cudaMemsetAsync(r->d_status, 0, sizeof(int32_t), s));
     if (with_cancel_and_events) {
-        RMS_CUDA(cudaHostAlloc((void **)&r->h_cancel, sizeof(int32_t), cudaHostAllocMapped));
+        RMS_TRY(take_cancel_flag(r));
         *r->h_cancel = 0;
         RMS_CUDA(cudaHostGetDevicePointer((void **)&r->d_cancel, r->h_cancel, 0));
         RMS_CUDA(cudaEventCreate(&r->ev_start));

@@ -6,6 +6,7 @@
 
 #include <algorithm>
 #include <atomic>
+#include <mutex>
 #include <string>
 #include <vector>
 
@@ -63,6 +64,14 @@ struct rms_sequence {
     int64_t pitch = 0;  // row pitch of d_wG64 and d_wG32
     double *d_dirs = nullptr, *d_b = nullptr, *d_bs = nullptr, *d_q = nullptr;
     double *d_trig = nullptr;  // azimuth table (FP64 form)
+    // Cancel flags of this sequence's runs: mapped host memory taken at the first
+    // run and freed with the sequence (taking and freeing one for every run was a
+    // quarter of the smallest run's 0.85 ms).  A run that finds all in use takes
+    // its own.
+    static constexpr int kCancelFlags = 64;
+    std::mutex flag_mu;
+    int32_t *h_flags = nullptr;
+    uint64_t flags_used = 0;
     std::atomic<int> refs{0};
 };
 
@@ -94,6 +103,7 @@ struct rms_run_handle {
     double *d_ro_partial = nullptr, *d_S = nullptr;
     int32_t *d_status = nullptr;
     int32_t *h_cancel = nullptr, *d_cancel = nullptr;
+    int32_t cancel_slot = -1;  // of the sequence's flags; -1: the run's own
     cudaEvent_t ev_start = nullptr, ev_end = nullptr;
     int32_t n_combo = 0, n_chunks = 0;
 };
