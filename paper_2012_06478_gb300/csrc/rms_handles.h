@@ -65,8 +65,8 @@ struct rms_sequence {
     double *d_dirs = nullptr, *d_b = nullptr, *d_bs = nullptr, *d_q = nullptr;
     double *d_trig = nullptr;  // azimuth table (FP64 form)
     // Cancel flags of this sequence's runs: mapped host memory taken at the first
-    // run and freed with the sequence (taking and freeing one for every run was a
-    // quarter of the smallest run's 0.85 ms).  A run that finds all in use takes
+    // run and freed with the sequence (taking and freeing one for every run was 0.34
+    // of the smallest run's 0.83 ms).  A run that finds all in use takes
     // its own.
     static constexpr int kCancelFlags = 64;
     std::mutex flag_mu;

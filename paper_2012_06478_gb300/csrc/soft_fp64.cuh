@@ -9,11 +9,11 @@
 // integer arithmetic (multiplies on the integer pipe, a single-precision
 // seed) gives the same bits at a fraction of the pipe time.
 //
-// Method: a reciprocal (or reciprocal square root) seed from single
-// precision, refined by Newton-Raphson iterations in fixed point (for the
-// reciprocal x' = x + x(1 - b x); for the square root q' = q + (X - q^2)/(2q)
-// with 1/(2q) from the seed), then an exact integer remainder that fixes the
-// last unit and decides the rounding -- the classical scheme of, e.g.,
+// Method: a reciprocal (or square root and its reciprocal) seed from single
+// precision, one Newton-Raphson step in fixed point (for the reciprocal x' = x +
+// x(1 - b x); for the square root q' = q + (X - q^2)/(2q) with 1/(2q) from the
+// seed), then exact integer remainders that bring the result to its last unit
+// and decide the rounding -- the classical scheme of, e.g.,
 // Muller et al., Handbook of Floating-Point Arithmetic (2nd ed., 2018),
 // ch. 4 (Newton-Raphson based division and square root) with the final
 // correction by the remainder.  Division and square root have no exact
@@ -103,13 +103,6 @@ __host__ __device__ __forceinline__ float sqrt_rn(float x)
 #endif
 }
 
-// floor(x * e / 2^64) rounded toward zero, x < 2^64 unsigned, e signed
-__host__ __device__ __forceinline__ int64_t smulhi(uint64_t x, int64_t e)
-{
-    const uint64_t m = mulhi(x, e < 0 ? (uint64_t)(-e) : (uint64_t)e);
-    return e < 0 ? -(int64_t)m : (int64_t)m;
-}
-
 // a / b for a and b known to be normal and positive, with a quotient known to be
 // normal (the caller's ranges guarantee it).
 __host__ __device__ __forceinline__ double div_normal(double a, double b)
@@ -119,26 +112,31 @@ __host__ __device__ __forceinline__ double div_normal(double a, double b)
     const uint64_t A = (ua & kMant) | kHidden, B = (ub & kMant) | kHidden;  // [2^52, 2^53)
     const bool ge = A >= B;
     const int32_t e = ea - eb + 1022 + (ge ? 1 : 0);  // biased exponent of the quotient
-    // x ~ 2^115 / B in (2^62, 2^63]: seed from the single-precision reciprocal
-    // of B's top 24 bits (relative error below 2^-22), exact as a shifted
-    // integer; then two Newton steps x += x e / 2^115, e = 2^115 - B x
+    // X0 ~ 2^76 / B in 24 bits, from the single-precision reciprocal of B's top 24
+    // (relative error below 2^-22)
     const float fr = rcp_rn((float)(uint32_t)(B >> 29));  // in (2^-24, 2^-23]
     const uint32_t fb = float_bits(fr);
-    uint64_t x = (uint64_t)((fb & 0x7FFFFFu) | 0x800000u) << ((fb >> 23) - 64u);  // fr 2^86
-#pragma unroll
-    for (int it = 0; it < 2; ++it) {
-        const uint64_t plo = B * x, phi = mulhi(B, x);  // B x < 2^116
-        // e = 2^115 - B x as a 128-bit two's-complement (ehi, elo); |e| < 2^94
-        const uint64_t elo = 0ULL - plo;
-        const int64_t ehi = (int64_t)(0x0008000000000000ULL - phi - (plo != 0ULL ? 1ULL : 0ULL));
-        const int64_t e51 = (int64_t)(((uint64_t)ehi << 13) | (elo >> 51));  // e / 2^51, |e51| < 2^43
-        x += (uint64_t)smulhi(x, e51);
-    }
-    // Q = floor(A 2^s / B), s = 52 (A >= B) or 53: from (A 2^11) x / 2^(126 - s),
-    // within one unit; the exact remainder fixes it
+    const uint32_t X0 = ((fb & 0x7FFFFFu) | 0x800000u) << ((fb >> 23) - 103u);  // fr 2^47
+    // one Newton step: X1 ~ 2^108 / B in (2^55, 2^56], relative error below 2^-44, with
+    // e = 2^55 - B X0 / 2^21, |e| < 2^33
+    const uint32_t Bh = (uint32_t)(B >> 21), Bl = (uint32_t)B & 0x1FFFFFu;
+    const int64_t e0 = (int64_t)(0x0080000000000000ULL - ((uint64_t)Bh * X0 + (((uint64_t)Bl * X0) >> 21)));
+    const uint64_t X1 = ((uint64_t)X0 << 32) + (uint64_t)(((int64_t)(int32_t)X0 * (int32_t)(e0 >> 3)) >> 20);
+    // Q = floor(A 2^s / B), s = 52 (A >= B) or 53: A X1 / 2^(108 - s) is within 2^9 of
+    // it; its exact remainder (below 2^62) over B brings it within one unit, and
+    // the remainder of that fixes it.  Products of 32-bit words throughout: a second
+    // Newton step in 64-bit ones takes twice as many
     const int s = ge ? 52 : 53;
-    uint64_t Q = mulhi(A << 11, x) >> (ge ? 10 : 9);
-    int64_t R = (int64_t)((A << s) - Q * B);  // exact: the true value lies in (-B, 2B)
+    const uint64_t As = A << s;  // mod 2^64
+    const uint32_t Ah = (uint32_t)(A >> 21), Al = (uint32_t)A << 11;  // A 2^11
+    const uint32_t Xh = (uint32_t)(X1 >> 25), Xl = (uint32_t)X1 << 7;  // X1 2^7
+    // (A 2^11) (X1 2^7) / 2^64, without the low words' product
+    const uint64_t P = (uint64_t)Ah * Xh + (((uint64_t)Ah * Xl) >> 32) + (((uint64_t)Al * Xh) >> 32);
+    uint64_t Q = P >> (ge ? 10 : 9);
+    int64_t R = (int64_t)(As - Q * B);
+    const int32_t dq = (int32_t)(((int64_t)(int32_t)(R >> 32) * (int32_t)(X1 >> 26)) >> 50);  // R X1 / 2^108
+    Q += (uint64_t)(int64_t)dq;
+    R -= (int64_t)dq * (int64_t)B;
     if (R < 0) {
         --Q;
         R += (int64_t)B;
@@ -245,40 +243,32 @@ __host__ __device__ __forceinline__ double sqrt_normal(double x)
     const int32_t E = ex - 1023;                        // x = M 2^(E - 52)
     const bool odd = (E & 1) != 0;
     // X = M 2^52 (E even) or M 2^53 (E odd): sqrt(x) = sqrt(X) 2^((E - odd)/2 - 52),
-    // sqrt(X) in [2^52, 2^53).  X as 128 bits:
+    // sqrt(X) in [2^52, 2^53)
     const int sh = odd ? 53 : 52;
-    const uint64_t Xlo = M << sh, Xhi = M >> (64 - sh);
-    // seed: X 2^-80 = M 2^(sh - 80) in [2^24, 2^26); q ~ sqrt(X) = sqrtf(.) 2^40,
-    // rq ~ 2^103 / sqrt(X) ~ 2^103 / q (for corrections D / (2 q))
-    const float xf = (float)(uint32_t)(M >> (80 - sh));  // truncated: relative error < 2^-24
-    const float sf = sqrt_rn(xf);                         // in [2^12, 2^13)
+    const uint64_t Xlo = M << sh;  // mod 2^64
+    // single precision's root of X 2^-80 = M 2^(sh - 80) in [2^24, 2^26) and its
+    // reciprocal: sqrt(X) ~ S 2^29 (relative error below 2^-23), 1 / 2 sqrt(X) ~ r 2^-77
+    const float sf = sqrt_rn((float)(uint32_t)(M >> (80 - sh)));  // in [2^12, 2^13)
     const uint32_t sb = float_bits(sf);
-    uint64_t q = (uint64_t)((sb & 0x7FFFFFu) | 0x800000u) << ((sb >> 23) - 110u);  // sf 2^40
-    const float rf = rcp_rn(sf);                          // in (2^-13, 2^-12]
-    const uint32_t rb = float_bits(rf);
-    const uint64_t rq = (uint64_t)((rb & 0x7FFFFFu) | 0x800000u) << ((rb >> 23) - 87u);  // rf 2^63
-    // two steps q += (X - q^2) / (2 q), the difference in 128 bits
-#pragma unroll
-    for (int it = 0; it < 2; ++it) {
-        const uint64_t slo = q * q, shi = mulhi(q, q);
-        const uint64_t dlo = Xlo - slo;
-        const int64_t dhi = (int64_t)(Xhi - shi - (Xlo < slo ? 1ULL : 0ULL));  // |X - q^2| < 2^87
-        const int64_t d40 = (int64_t)(((uint64_t)dhi << 24) | (dlo >> 40));   // (X - q^2) / 2^40
-        // (X - q^2)/(2q) = d40 2^40 / (2 q) ~ d40 rq 2^40 / 2^104 = d40 rq / 2^64
-        q += (uint64_t)smulhi(rq, d40);
-    }
-    // exact remainder R = X - q^2 (mod 2^64; the true value is far inside);
-    // bring q to floor(sqrt(X)): 0 <= R <= 2q
+    const uint32_t S = ((sb & 0x7FFFFFu) | 0x800000u) << ((sb >> 23) - 139u);  // sf 2^11
+    const uint32_t rb = float_bits(rcp_rn(sf));                                // in (2^-13, 2^-12]
+    const int32_t r = (int32_t)(((rb & 0x7FFFFFu) | 0x800000u) << ((rb >> 23) - 114u));  // rf 2^36
+    // q1 = S 2^29 + (X - S^2 2^58) / 2 sqrt(X), the difference exact in units of 2^52 (below
+    // 2^32 of them): within 2^8 of sqrt(X)
+    const int64_t D0 = (int64_t)((M << (sh - 52)) - (((uint64_t)S * S) << 6));
+    uint64_t q = ((uint64_t)S << 29) + (uint64_t)(((int64_t)(int32_t)(D0 >> 2) * r) >> 23);
+    // its exact remainder (below 2^62) over 2 sqrt(X) brings it to floor(sqrt(X)) or a
+    // unit beside it, and the remainder of that, in [0, 2q] for the floor, fixes it
     int64_t R = (int64_t)(Xlo - q * q);
-#pragma unroll
-    for (int it = 0; it < 2; ++it) {
-        if (R < 0) {
-            R += (int64_t)(2 * q - 1);
-            --q;
-        } else if (R > (int64_t)(2 * q)) {
-            R -= (int64_t)(2 * q + 1);
-            ++q;
-        }
+    const int32_t dq = (int32_t)(((int64_t)(int32_t)(R >> 32) * r) >> 45);
+    R -= (int64_t)dq * (int64_t)(2 * q + (uint64_t)(int64_t)dq);
+    q += (uint64_t)(int64_t)dq;
+    if (R < 0) {
+        R += (int64_t)(2 * q - 1);
+        --q;
+    } else if (R > (int64_t)(2 * q)) {
+        R -= (int64_t)(2 * q + 1);
+        ++q;
     }
     // round to nearest: sqrt(X) >= q + 1/2 iff X - q^2 > q (no ties)
     const uint64_t up = (uint64_t)R > q ? 1ULL : 0ULL;

@@ -195,22 +195,11 @@ __device__ __forceinline__ double odd_scaled(uint32_t mag, bool neg, int e2)
 // IEEE result of a product of doubles whose exact value is N 2^-64.
 __device__ __forceinline__ double u64_scaled_rn(unsigned long long N)
 {
-    const int p = 63 - __clzll((long long)N);
-    int e = p - 64;
-    unsigned long long q;
-    if (p <= 52) {
-        q = N << (52 - p);
-    } else {
-        const int sh = p - 52;
-        q = N >> sh;
-        const unsigned long long rem = N & ((1ULL << sh) - 1ULL), half = 1ULL << (sh - 1);
-        if (rem > half || (rem == half && (q & 1ULL))) ++q;
-        if (q >> 53) {
-            q >>= 1;
-            ++e;
-        }
-    }
-    return __longlong_as_double((long long)(((unsigned long long)(e + 1023) << 52) | (q & 0x000FFFFFFFFFFFFFULL)));
+    // the leading one to bit 63: 53 bits kept, 11 below them
+    const int z = __clzll((long long)N);
+    const unsigned long long t = (unsigned long long)N << z, m = t >> 11;
+    const unsigned long long up = ((uint32_t)t & 0x7FFu) + ((uint32_t)m & 1u) > 0x400u ? 1ULL : 0ULL;
+    return __longlong_as_double((long long)(((unsigned long long)(1021 - z) << 52) + m + up));
 }
 
 // UNROLL: all products side by side (the four-lane kernel, bound by their latency).
