@@ -74,6 +74,20 @@ __device__ __forceinline__ double dclamp01(double x)
     return b > 0x3FF0000000000000LL ? 1.0 : x;
 }
 
+// -x by its sign bit, in assembly: the compiler negates a double with an
+// addition, a slot of the FP64 pipe (a dozen of a step's 44).
+__device__ __forceinline__ double dneg(double x)
+{
+    int hi = __double2hiint(x);
+    asm("xor.b32 %0, %0, 0x80000000;" : "+r"(hi));
+    return __hiloint2double(hi, __double2loint(x));
+}
+__device__ __forceinline__ double negated(double x) { return dneg(x); }
+__device__ __forceinline__ float negated(float x) { return -x; }
+// x != 0, NaNs among them
+__device__ __forceinline__ bool nonzero(double x) { return (dbits(x) << 1) != 0; }
+__device__ __forceinline__ bool nonzero(float x) { return x != 0.0f; }
+
 // Sec. 2.2 item 2, the direction.  z = 1 - 2u is uniform on [-1, 1] for a
 // uniform point of the sphere (Archimedes); the azimuth is
 // phi = 2 pi (x1 + 1/2) 2^-32.  Its sine and cosine come from Taylor
@@ -89,8 +103,8 @@ __device__ __forceinline__ void octant_map(uint32_t oct, double cs, double sn, d
     const bool negx = ((oct + 2u) >> 2) & 1u;  // octants 2..5
     const bool negy = (oct >> 2) & 1u;         // octants 4..7
     const double a = swap ? sn : cs, b = swap ? cs : sn;
-    cx = negx ? -a : a;
-    sy = negy ? -b : b;
+    cx = negx ? dneg(a) : a;
+    sy = negy ? dneg(b) : b;
 }
 
 // The hardware FP64 operations, for the operands the integer-ALU versions
@@ -243,7 +257,7 @@ __device__ __forceinline__ void direction_from(uint32_t x0, uint32_t x1, const d
         for (int i = 0; i < 2; ++i) {
             cs = sn;
             sn = mul_normal(p, ce) - mul_normal(q, se);
-            const double m = -p;
+            const double m = dneg(p);
             p = q;
             q = m;
         }
@@ -616,7 +630,7 @@ __device__ __forceinline__ void walk_block(const Geometry &g, const Tables<Real>
         bool graded;
         if constexpr (NS == 1) {
             wg = __ldg(t.wG + (k - 1));
-            graded = wg != Real(0);
+            graded = nonzero(wg);
         } else {
             graded = (__ldg(t.flags + (k - 1)) & 1u) != 0u;
         }
@@ -713,8 +727,8 @@ __device__ __forceinline__ void walk_block(const Geometry &g, const Tables<Real>
 #pragma unroll
                     for (int a = 0; a < 3; ++a)
                         if (a == best) {
-                            n[a] = -n[a];
-                            d[a] = -d[a];
+                            n[a] = negated(n[a]);
+                            d[a] = negated(d[a]);
                         }
                 }
                 return false;

@@ -75,7 +75,7 @@ walk_quad_kernel(Geometry g, Tables<double> t, WalkerState<double> st, RunCtl ct
         bool graded;
         if constexpr (NS == 1) {
             wg = __ldg(t.wG + (k - 1));
-            graded = wg != kZero;
+            graded = nonzero(wg);
         } else {
             graded = (__ldg(t.flags + (k - 1)) & 1u) != 0u;
         }
@@ -162,8 +162,8 @@ walk_quad_kernel(Geometry g, Tables<double> t, WalkerState<double> st, RunCtl ct
                         } else {  // reflected: stays in its voxel, at the face
                             nv = v;
                             if (mine) {
-                                n = -n;
-                                d = -d;
+                                n = dneg(n);
+                                d = dneg(d);
                                 o = up ? 1.0 : 0.0;
                                 di -= up ? 1 : -1;
                             }
