@@ -75,16 +75,6 @@ __host__ __device__ __forceinline__ uint32_t float_bits(float x)
 #endif
 }
 
-// high 64 bits of the 128-bit product a*b
-__host__ __device__ __forceinline__ uint64_t mulhi(uint64_t a, uint64_t b)
-{
-#ifdef __CUDA_ARCH__
-    return __umul64hi(a, b);
-#else
-    return (uint64_t)(((unsigned __int128)a * b) >> 64);
-#endif
-}
-
 // single-precision reciprocal and square root, correctly rounded on both sides
 __host__ __device__ __forceinline__ float rcp_rn(float x)
 {
@@ -168,6 +158,19 @@ __host__ __device__ __forceinline__ bool div_pos(double a, double b, double &q)
     return true;
 }
 
+// A B of two 53-bit significands in two words: their high words have 21 bits, so
+// the middle products add up without a carry -- four products of 32-bit words
+// with their additions, where separate low and high products take seven and the
+// carries.
+__host__ __device__ __forceinline__ void mul_significands(uint64_t A, uint64_t B, uint64_t &lo, uint64_t &hi)
+{
+    const uint32_t a0 = (uint32_t)A, a1 = (uint32_t)(A >> 32), b0 = (uint32_t)B, b1 = (uint32_t)(B >> 32);
+    const uint64_t p = (uint64_t)a0 * b0;
+    const uint64_t m = (uint64_t)a0 * b1 + ((uint64_t)a1 * b0 + (p >> 32));
+    hi = (uint64_t)a1 * b1 + (m >> 32);
+    lo = (m << 32) | (uint32_t)p;
+}
+
 // The product of the significands of a and b rounded to 53 bits, given the
 // biased exponent e of the result: the 106-bit product is exact in two words,
 // brought to [2^105, 2^106) (doubled when below), so that the 53 kept bits
@@ -214,7 +217,8 @@ __host__ __device__ __forceinline__ bool mul_rn(double a, double b, double &p)
     const int32_t ea = (int32_t)((ua >> 52) & 0x7FFu), eb = (int32_t)((ub >> 52) & 0x7FFu);
     if ((uint32_t)(ea - 1) >= 0x7FEu || (uint32_t)(eb - 1) >= 0x7FEu) return false;
     const uint64_t A = (ua & kMant) | kHidden, B = (ub & kMant) | kHidden;
-    const uint64_t lo = A * B, hi = mulhi(A, B);  // A B in [2^104, 2^106)
+    uint64_t lo, hi;  // A B in [2^104, 2^106)
+    mul_significands(A, B, lo, hi);
     const bool top = (hi >> 41) != 0ULL;          // A B >= 2^105
     const int32_t e = ea + eb - 1023 + (top ? 1 : 0);
     if ((uint32_t)(e - 1) >= 0x7FEu) return false;
@@ -229,7 +233,8 @@ __host__ __device__ __forceinline__ double mul_normal(double a, double b)
     const uint64_t ua = bits_of(a), ub = bits_of(b);
     const int32_t ea = (int32_t)((ua >> 52) & 0x7FFu), eb = (int32_t)((ub >> 52) & 0x7FFu);
     const uint64_t A = (ua & kMant) | kHidden, B = (ub & kMant) | kHidden;
-    const uint64_t lo = A * B, hi = mulhi(A, B);
+    uint64_t lo, hi;
+    mul_significands(A, B, lo, hi);
     const bool top = (hi >> 41) != 0ULL;
     return mul_core(ua, ub, lo, hi, top, ea + eb - 1023 + (top ? 1 : 0));
 }

@@ -99,12 +99,12 @@ __device__ __forceinline__ bool nonzero(float x) { return x != 0.0f; }
 // warp ever loops on a rejection.
 __device__ __forceinline__ void octant_map(uint32_t oct, double cs, double sn, double &cx, double &sy)
 {
-    const bool swap = ((oct + 1u) >> 1) & 1u;  // octants 1, 2, 5, 6
-    const bool negx = ((oct + 2u) >> 2) & 1u;  // octants 2..5
-    const bool negy = (oct >> 2) & 1u;         // octants 4..7
+    const bool swap = ((oct + 1u) >> 1) & 1u;                      // octants 1, 2, 5, 6
+    const int negx = (int)(((oct + 2u) << 29) & 0x80000000u);      // octants 2..5
+    const int negy = (int)((oct << 29) & 0x80000000u);             // octants 4..7
     const double a = swap ? sn : cs, b = swap ? cs : sn;
-    cx = negx ? dneg(a) : a;
-    sy = negy ? dneg(b) : b;
+    cx = __hiloint2double(__double2hiint(a) ^ negx, __double2loint(a));
+    sy = __hiloint2double(__double2hiint(b) ^ negy, __double2loint(b));
 }
 
 // The hardware FP64 operations, for the operands the integer-ALU versions
