@@ -301,19 +301,16 @@ __device__ __forceinline__ void direction_from(uint32_t x0, uint32_t x1, const d
     const float z = -((float)(int32_t)(x0 ^ 0x80000000u) + 0.5f) * 0x1p-31f;
     const float rr = (1.0f - z) * (1.0f + z);
     const float r = rr * rsqrt_normal(rr);
-    const uint32_t oct = x1 >> 29;
-    uint32_t m = x1 & 0x1FFFFFFFu;
-    if (oct & 1u) m = 0x1FFFFFFFu - m;
+    // the octant's fold, swap and signs from the word's own bits
+    const uint32_t m = (x1 ^ (uint32_t)((int32_t)(x1 << 2) >> 31)) & 0x1FFFFFFFu;  // odd octants from their end
     const float th = ((float)m + 0.5f) * (0x1p-29f * 0.785398163f);
     const float t = th * th;
     const float sn = th + (th * t) * (-1.0f / 6.0f + t * (1.0f / 120.0f + t * (-1.0f / 5040.0f)));
     const float cs = 1.0f + t * (-0.5f + t * (1.0f / 24.0f + t * (-1.0f / 720.0f + t * (1.0f / 40320.0f))));
-    const bool swap = ((oct + 1u) >> 1) & 1u;
-    const bool negx = ((oct + 2u) >> 2) & 1u;
-    const bool negy = (oct >> 2) & 1u;
+    const bool swap = ((x1 + 0x20000000u) & 0x40000000u) != 0u;  // octants 1, 2, 5, 6
     const float a = swap ? sn : cs, b = swap ? cs : sn;
-    n[0] = r * (negx ? -a : a);
-    n[1] = r * (negy ? -b : b);
+    n[0] = r * __uint_as_float(__float_as_uint(a) ^ ((x1 + 0x40000000u) & 0x80000000u));  // octants 2..5
+    n[1] = r * __uint_as_float(__float_as_uint(b) ^ (x1 & 0x80000000u));                  // octants 4..7
     n[2] = z;
 }
 
@@ -878,9 +875,9 @@ __device__ __forceinline__ void walk_block(const Geometry &g, const Tables<Real>
                     const int best = b2 ? 2 : (b1 ? 1 : 0);
                     const bool up = (b2 ? d[2] : (b1 ? d[1] : d[0])) > Real(0);
                     const int32_t sb = b2 ? stride[2] : (b1 ? stride[1] : 1);
-                    int32_t nv = up ? v + sb : v - sb;
-                    const uint32_t bit = (b2 ? kFaceZ : (b1 ? kFaceY : kFaceX)) << (up ? 3 : 0);
                     const int32_t inc = up ? 1 : -1;
+                    int32_t nv = v + inc * sb;
+                    const uint32_t bit = (b2 ? kFaceZ : (b1 ? kFaceY : kFaceX)) << (up ? 3 : 0);
                     const Real at = up ? Real(0) : Real(1);
 #pragma unroll
                     for (int a = 0; a < 3; ++a) {
