@@ -6,21 +6,26 @@
 // and by walk_reject_fp{64,32}.cu and walk_mt_fp{64,32}.cu for the other
 // particle-membrane interactions and for absorbing membranes.
 //
-// One thread owns one walker for a slice of steps; its whole state stays in
-// registers for the slice and goes back to global memory (structure of
-// arrays, coalesced) at the end.  Per step and walker the only memory
-// traffic is one byte for each voxel entered -- its face bits, which say
-// whether each of the voxel's faces leads into the same label (Sec. 2.1.1: the
-// volume is the lookup table) -- at a membrane the label across it and the
-// threshold of the label pair (and its saturation threshold, with absorbing
-// membranes), and warp-uniform broadcasts of the waveform.
+// One thread owns one walker for a slice of steps; its state stays in registers
+// (the plain form's phases and start offsets in shared memory) for the slice and
+// goes back to global memory (structure of arrays, coalesced) at the end.  Per
+// step and walker the only memory traffic is one byte for each voxel entered --
+// its face bits, which say whether each of the voxel's faces leads into the same
+// label (Sec. 2.1.1: the volume is the lookup table) -- at a membrane the label
+// across it and the threshold of the label pair (and its saturation threshold,
+// with absorbing membranes), and warp-uniform broadcasts of the waveform.
 //
-// What bounds it: the FP32 step issues (323 warp-instructions per warp-step on
-// 200x200x400 axons, issue slots 74 % used, ALU pipe 65 %).  Deciding the
+// What bounds it: the FP32 step issues (332 warp-instructions per warp-step on
+// 200x200x400 axons, issue slots 77 % used, ALU pipe 64 %).  Deciding the
 // events from face bits instead of a label gather with wrapped coordinates,
 // with selects in place of branches, the step's tables and weights read ahead
 // and nothing done for relaxation when no label relaxes took 1e6 walkers x
-// 2000 steps from 27.4 ms (428 warp-instructions) to 21.8 ms, the same bits.
+// 2000 steps from 27.4 ms (428 warp-instructions) to 21.8 ms; packed phase sums
+// and octants without selects took the call of 10 000 steps from 112.6 ms to
+// 108.4; the same bits.  The plain form's step uses the ALU, the integer
+// products' and the FP64 pipe alike (72, 72 and 68 %, issue 77 %): 170 ms for
+// the same launch, 269 before the loops over axes, unchecked arithmetic and
+// shorter products, quotients and roots.
 #pragma once
 
 #include <cstdint>
