@@ -429,7 +429,7 @@ rms_status rms_philox4x32_10(const uint32_t *ctr, const uint32_t *key, int64_t n
 
 /* The same read-out as rms_run's in the plain FP64 form (S = sum alpha
  * e^{-i phi} / sum alpha, phi = q g.Phi_s, q = sqrt(b / b_s), alpha =
- * exp(-A), every term in FP64) over walker data the caller holds.  Every pointer is a DEVICE pointer of the current device:
+ * exp(-A), every term within 2^-52 of alpha's largest) over walker data the caller holds.  Every pointer is a DEVICE pointer of the current device:
  *   phase     : n_walkers*n_shapes*3 doubles, row-major (walker, shape, axis),
  *               the layout rms_read_walkers returns
  *   A         : n_walkers doubles, exponent of Eq. 5

@@ -78,3 +78,22 @@ def test_values_that_are_not_finite():
     assert np.isnan(got[0, 1]).all()
     got, asum = _readout(np.zeros((1000, 1, 3)), np.full(1000, np.inf), bs, dirs, b)
     assert asum == 0.0 and np.isnan(got).all()
+
+
+def test_under_capture():
+    import torch
+    from paper_2012_06478_gb300 import _lib
+    rng = np.random.default_rng(4)
+    arrays = rng.normal(size=(1000, 1, 3)), rng.uniform(size=1000), np.ones(1), np.eye(3), np.array([0.0, 2.0])
+    want, _ = _readout(*arrays)  # the first call, before the capture
+    t = [torch.from_numpy(np.ascontiguousarray(x)).cuda() for x in arrays]
+    re, im = torch.zeros((2, 6), dtype=torch.float64, device="cuda").unbind(0)
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph):
+        rc = _lib.lib.rms_readout_noalloc(t[0].data_ptr(), t[1].data_ptr(), 1000, 1, t[2].data_ptr(), 3, t[3].data_ptr(),
+                                          2, t[4].data_ptr(), re.data_ptr(), im.data_ptr(), None,
+                                          C.c_void_p(torch.cuda.current_stream().cuda_stream))
+        assert rc == _lib.RMS_OK, _lib.last_error()
+    graph.replay()
+    torch.cuda.synchronize()
+    np.testing.assert_array_equal(re.cpu().numpy() + 1j * im.cpu().numpy(), want.ravel())
