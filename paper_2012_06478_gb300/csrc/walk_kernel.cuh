@@ -192,12 +192,6 @@ __device__ __forceinline__ double over(double a, double b)
     }
 }
 
-template <bool SANE = false>
-__device__ __forceinline__ float times_any(float a, float b)
-{
-    return a * b;
-}
-
 // Exact doubles built from their bits on the integer ALU, so that values
 // which need no rounding do not occupy GB300's narrow FP64 pipe.
 // k * 2^e2 for an odd |k| < 2^32: no rounding, the same bits as converting k
