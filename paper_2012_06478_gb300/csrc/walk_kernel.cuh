@@ -568,7 +568,8 @@ __device__ __forceinline__ void walk_block(const Geometry &g, const Tables<Real>
         for (int i = 0; i < kRoundKeys; ++i) rk[i] = ctl.rk[i];
     }
     // threads beyond the last walker walk a copy of it and write nothing: no
-    // branch on it in the step loop
+    // branch on it in the step loop, and what a copy reports (status) is what its
+    // walker reports
     const bool active = block * kWalkBlock + threadIdx.x < ctl.n_walkers;
     const int64_t li = active ? block * kWalkBlock + threadIdx.x : ctl.n_walkers - 1;
     // the walker in this slot: its id picks its random streams (RMS_MORTON
@@ -616,6 +617,9 @@ __device__ __forceinline__ void walk_block(const Geometry &g, const Tables<Real>
         }
     }
     int32_t next_rec = rec < ctl.n_rec ? __ldg(t.rec_step + rec) : INT32_MAX;
+    // the copies of the last walker have read its state before its own thread, in
+    // another warp, writes it back at the end of the slice
+    __syncthreads();
 
     // a 32-bit step counter (n_steps <= 2e9): uniform 32-bit arithmetic per
     // step (measured 0.8 % faster than 64-bit on the FP32 step)

@@ -69,6 +69,7 @@ walk_quad_kernel(Geometry g, Tables<double> t, WalkerState<double> st, RunCtl ct
 #pragma unroll
     for (int s = 0; s < NS; ++s) ph[s] = s < ctl.n_shapes ? st.phase[((int64_t)s * 3 + a) * ctl.n_walkers + li] : kZero;
     int32_t next_rec = rec < ctl.n_rec ? __ldg(t.rec_step + rec) : INT32_MAX;
+    __syncthreads();  // the copies of the last walker have read it before its own lanes write it back
 
     for (int32_t k = (int32_t)k_begin + 1; k <= (int32_t)k_end; ++k) {
         double wg = kZero;
