@@ -23,8 +23,8 @@
 // normal, with a normal result -- and returns false for anything else, so
 // the caller falls back to the hardware operation for zeros, subnormals,
 // infinities, NaNs and out-of-range results.  Host and device share the
-// code: the host build (for the host-side checks) replaces the two device
-// intrinsics by their exact definitions.
+// code: the host build (for the host-side checks) replaces the single-precision
+// seeds, the funnel shift and the carry chain by their exact definitions.
 #pragma once
 
 #include <cstdint>
@@ -171,23 +171,21 @@ __host__ __device__ __forceinline__ void mul_significands(uint64_t A, uint64_t B
     lo = (m << 32) | (uint32_t)p;
 }
 
-// The product of the significands of a and b rounded to 53 bits, given the
-// biased exponent e of the result: the 106-bit product is exact in two words,
-// brought to [2^105, 2^106) (doubled when below), so that the 53 kept bits
-// and the 53 below them sit at fixed places; rounding is to nearest with ties
-// to even (products do have ties).
-__host__ __device__ __forceinline__ double mul_core(uint64_t ua, uint64_t ub, uint64_t lo, uint64_t hi, bool top,
-                                                    int32_t e)
+// The upper word of (hi 2^32 + lo) 2^s, s < 32.
+__host__ __device__ __forceinline__ uint32_t funnel_left(uint32_t lo, uint32_t hi, uint32_t s)
 {
 #ifdef __CUDA_ARCH__
-    // The kept bits and, left-aligned, the ones below them by funnel shifts; the
-    // carry of the latter plus one half -- less one unit where the kept part is
-    // even -- is the rounding (10 operations of the ALU in place of 17).
-    const uint32_t s = top ? 11u : 12u;
-    const uint32_t l0 = (uint32_t)lo, l1 = (uint32_t)(lo >> 32), h0 = (uint32_t)hi, h1 = (uint32_t)(hi >> 32);
-    const uint32_t m0 = __funnelshift_l(l1, h0, s), m1 = __funnelshift_l(h0, h1, s);
-    const uint32_t r0 = l0 << s, r1 = __funnelshift_l(l0, l1, s), odd = m0 & 1u;
-    const uint32_t head = ((uint32_t)((ua ^ ub) >> 32) & 0x80000000u) | ((uint32_t)(e - 1) << 20);
+    return __funnelshift_l(lo, hi, s);
+#else
+    return (uint32_t)(((((uint64_t)hi << 32) | lo) << s) >> 32);
+#endif
+}
+
+// m1 2^32 + m0 + head 2^32, plus the carry of (r1 2^32 + r0) + (x1 2^32 + x0).
+__host__ __device__ __forceinline__ double add_carry_of(uint32_t r0, uint32_t r1, uint32_t x0, uint32_t x1, uint32_t m0,
+                                                        uint32_t m1, uint32_t head)
+{
+#ifdef __CUDA_ARCH__
     uint32_t p0, p1;
     asm("{\n\t.reg .u32 t;\n\t"
         "add.cc.u32 t, %2, %3;\n\t"
@@ -195,17 +193,32 @@ __host__ __device__ __forceinline__ double mul_core(uint64_t ua, uint64_t ub, ui
         "addc.cc.u32 %0, %6, 0;\n\t"
         "addc.u32 %1, %7, %8;\n\t}"
         : "=r"(p0), "=r"(p1)
-        : "r"(r0), "r"(odd - 1u), "r"(r1), "r"(odd + 0x7FFFFFFFu), "r"(m0), "r"(m1), "r"(head));
+        : "r"(r0), "r"(x0), "r"(r1), "r"(x1), "r"(m0), "r"(m1), "r"(head));
     return __hiloint2double((int)p1, (int)p0);
 #else
-    const uint64_t hn = top ? hi : (hi << 1) | (lo >> 63);
-    const uint64_t ln = top ? lo : lo << 1;
-    const uint64_t M = (hn << 11) | (ln >> 53);  // in [2^52, 2^53)
-    const uint64_t rem = ln & 0x001FFFFFFFFFFFFFULL;
-    // up iff rem > 2^52, or rem == 2^52 and M odd
-    const uint64_t up = rem + (M & 1ULL) > 0x0010000000000000ULL ? 1ULL : 0ULL;
-    return double_of(((ua ^ ub) & 0x8000000000000000ULL) | ((((uint64_t)(e - 1)) << 52) + M + up));
+    const uint64_t c0 = ((uint64_t)r0 + x0) >> 32, c1 = ((uint64_t)r1 + x1 + c0) >> 32;
+    const uint64_t p0 = (uint64_t)m0 + c1;
+    const uint32_t p1 = m1 + head + (uint32_t)(p0 >> 32);
+    return double_of(((uint64_t)p1 << 32) | (uint32_t)p0);
 #endif
+}
+
+// The product of the significands of a and b rounded to 53 bits, given the
+// biased exponent e of the result: the 106-bit product is exact in two words,
+// `top` says that it is at least 2^105; rounding is to nearest with ties to even
+// (products do have ties).  The kept bits and, left-aligned, the ones below them
+// come from funnel shifts; the carry of the latter plus one half -- less one unit
+// where the kept part is even -- is the rounding (10 operations of the ALU in
+// place of 17 for a comparison).
+__host__ __device__ __forceinline__ double mul_core(uint64_t ua, uint64_t ub, uint64_t lo, uint64_t hi, bool top,
+                                                    int32_t e)
+{
+    const uint32_t s = top ? 11u : 12u;
+    const uint32_t l0 = (uint32_t)lo, l1 = (uint32_t)(lo >> 32), h0 = (uint32_t)hi, h1 = (uint32_t)(hi >> 32);
+    const uint32_t m0 = funnel_left(l1, h0, s), m1 = funnel_left(h0, h1, s);
+    const uint32_t r0 = l0 << s, r1 = funnel_left(l0, l1, s), odd = m0 & 1u;
+    const uint32_t head = ((uint32_t)((ua ^ ub) >> 32) & 0x80000000u) | ((uint32_t)(e - 1) << 20);
+    return add_carry_of(r0, r1, odd - 1u, odd + 0x7FFFFFFFu, m0, m1, head);
 }
 
 // a * b, both finite, normal and of any sign, with a normal product
