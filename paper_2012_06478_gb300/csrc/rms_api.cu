@@ -150,7 +150,9 @@ __global__ void label_tables_kernel(int32_t L, const double *D, const double *T2
     const double ds = sqrt((6.0 * D[c]) * dt);
     const double s = ds / voxel;
     s64[c] = s;
-    s32[c] = (float)s;
+    // 2^-78 voxels in place of less: the FP32 step divides by 2^-42 of it and more, all
+    // normal numbers, and no walker gets anywhere by either
+    s32[c] = s > 0.0 ? fmaxf((float)s, kMinStepF) : 0.0f;
     const double r2 = isinf(T2[c]) ? 0.0 : dt / T2[c];
     const double r1 = isinf(T1[c]) ? 0.0 : dt / T1[c];
     dtR64[c] = r2;

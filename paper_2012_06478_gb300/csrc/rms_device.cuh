@@ -143,6 +143,9 @@ struct WalkerState {
     int32_t *wid;      // walker (relative to the run's first) in each slot, or nullptr: the slot's index
 };
 
+// The FP32 form's shortest step length, in voxels (but for 0).
+constexpr float kMinStepF = 0x1p-78f;
+
 // Quotients n / d for 0 <= n < 2^31 by a multiplication: with 2^(l-1) < d <=
 // 2^l, mul = ceil(2^(31+l) / d) < 2^32 and n mul >> (31 + l) is the quotient,
 // since the excess mul d - 2^(31+l) < 2^l adds less than n 2^l < 2^(31+l) to

@@ -274,10 +274,11 @@ __device__ __forceinline__ void direction_from(uint32_t x0, uint32_t x1, const d
     n[2] = z;
 }
 
-// a / b for b > 0 as a times the hardware reciprocal (its error is within 1 ulp),
-// infinite for b = 0 -- the bits of __fdividef for every normal b, without its
-// rescaling of subnormal divisors: the FP32 step's divisors |d| are zero or
-// above 1e-13 of the step length.  Likewise the reciprocal square root.
+// a times the approximate reciprocal of b >= 0 (within 1 ulp; a subnormal b counts
+// as 0, whose reciprocal is infinite), and the approximate reciprocal square root:
+// one instruction each.  The divisors |d| of the FP32 step are 0 or normal: a
+// direction's components are 0 or above 2^-42, and a label's step length is 0 or at
+// least kMinStepF voxels.
 __device__ __forceinline__ float mul_rcp(float a, float b)
 {
     float r;
