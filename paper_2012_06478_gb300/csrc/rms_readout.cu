@@ -60,30 +60,6 @@ __device__ __forceinline__ int top_exponent(double a, double b)
     return (int)(__reduce_max_sync(0xffffffffu, max(u, v)) >> 20);
 }
 
-// Sums of at most 64 pairs of numbers below 1: each is split at 2^-16 and 2^-33
-// by adding it to a number of fixed exponent, whose last place that is, so that
-// all sums but the last level's (below 2^-28) are exact.  Seven packed
-// additions, in place of two on the FP64 pipe.
-struct SplitSum {
-    static constexpr float kTop = 192.0f, kMid = 0x1.8p-10f;
-    F2 a = pair_of(kTop, kTop), b = pair_of(kMid, kMid), c = pair_of(0.0f, 0.0f);
-    __device__ __forceinline__ void add(F2 x)
-    {
-        const F2 ta = a + x;
-        x = x - (ta - a);
-        a = ta;
-        const F2 tb = b + x;
-        c = c + (x - (tb - b));
-        b = tb;
-    }
-    // one sum with 48 fraction bits
-    static __device__ __forceinline__ int64_t fixed(float a, float b, float c)
-    {
-        return ((int64_t)(__float_as_int(a) - __float_as_int(kTop)) << 32) +
-               ((int64_t)(__float_as_int(b) - __float_as_int(kMid)) << 15) + __float2int_rn(c * 0x1p48f);
-    }
-};
-
 // g.Phi of walker j's staged phases (the FP32 form's with their compensations).
 __device__ __forceinline__ double dot(const double *v, int, int j, const double *g)
 {
