@@ -21,7 +21,7 @@ __device__ const fix::Octant g_octant = fix::octant_table();
 constexpr int kTile = 64;         // walkers staged at a time: their exact sums fit 64 bits
 constexpr int kMaxThreads = 512;
 constexpr int kMaxPairs = 130;    // (shape, direction) pairs of one block's combinations, at most
-constexpr int64_t kMostWalkers = 16384;  // of a chunk, plain form
+constexpr int64_t kMostWalkers = 16384;  // of a chunk, but for a limit on chunks
 constexpr int kMinWalkers = 256;  // fewer: floating-point terms (their roundings are not averaged out)
 
 // The forms' staged numbers: the plain form's terms are integers; the FP32
@@ -109,7 +109,8 @@ constexpr size_t smem_bytes(int S, int pitch)
            sizeof(typename F::Phase) * kTile * pitch + sizeof(int) * pitch;
 }
 
-// Grid: x a group of p.cpb combinations, y a chunk of p.per walkers.  A thread
+// Grid: x a group of p.cpb combinations, y and z a chunk of p.per walkers (the groups of
+// a chunk run together and share its walkers in the L2).  A thread
 // has one combination and every p.nsub-th walker of the chunk.
 //
 // What bounds it: issue, and the pipe of the 32-bit products (plain form, 1e6
@@ -140,6 +141,8 @@ __global__ void __launch_bounds__(kMaxThreads, Form<Real>::kBlocks) readout_fixe
     if constexpr (kF64)
         for (int k = threadIdx.x; k < fix::kAngles; k += blockDim.x) table[k] = fix::angle_of(g_octant, k);
 
+    const int64_t chunk = (int64_t)blockIdx.z * gridDim.y + blockIdx.y;
+    if (chunk >= p.n_chunks) return;  // block-uniform
     const int64_t c0 = (int64_t)blockIdx.x * p.cpb;
     const int n_here = (int)min((int64_t)p.cpb, p.n_combo - c0);
     const int pair0 = (int)(c0 / p.n_b), n_pairs = (int)((c0 + n_here - 1) / p.n_b) - pair0 + 1;
@@ -158,7 +161,7 @@ __global__ void __launch_bounds__(kMaxThreads, Form<Real>::kBlocks) readout_fixe
     }
     const int64_t Q = fix::turns_of(q);
 
-    const int64_t w0 = (int64_t)blockIdx.y * p.per, w1 = min(p.W, w0 + p.per);
+    const int64_t w0 = chunk * p.per, w1 = min(p.W, w0 + p.per);
     const auto stage = [&](int64_t base, Real *to) {  // asynchronous copy of a tile's walkers
         const int nt = (int)min((int64_t)kTile, w1 - base);
         for (int e = threadIdx.x; e < rows * kTile; e += blockDim.x) {
@@ -178,14 +181,15 @@ __global__ void __launch_bounds__(kMaxThreads, Form<Real>::kBlocks) readout_fixe
     };
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, n_warps = (blockDim.x + 31) >> 5;
     double re = 0.0, im = 0.0, asum = 0.0;
-    // FP32 form: the sums of the tiles so far that had their alphas' exponent, 48 fraction bits
+    // FP32 form: the sums of the tiles so far that had their alphas' exponent, 48 fraction
+    // bits; a tile's is at most 64, a chunk's at most 2^62 in all (launch_readout)
     [[maybe_unused]] int64_t re48 = 0, im48 = 0;
-    [[maybe_unused]] int ea48 = 0, tiles48 = 0;
+    [[maybe_unused]] int ea48 = 0;
     [[maybe_unused]] const auto flush = [&] {
         const double scale = __longlong_as_double((long long)(ea48 - 47) << 52);  // 2^(ea48 - 1022 - 48)
         re += (double)re48 * scale;
         im -= (double)im48 * scale;
-        re48 = im48 = tiles48 = 0;
+        re48 = im48 = 0;
     };
     stage(w0, raw);
     int at = 0;
@@ -281,8 +285,8 @@ __global__ void __launch_bounds__(kMaxThreads, Form<Real>::kBlocks) readout_fixe
                         sincosf(qq * X[j * p.pitch + pair], &sn, &cs);
                         sum.add(pair_of(alF[j] * cs, alF[j] * sn));
                     }
-                    if (ea != ea48 || tiles48 == 256) {
-                        if (tiles48) flush();
+                    if (ea != ea48) {
+                        if (ea48) flush();
                         ea48 = ea;
                     }
                     // a phase that is not finite makes the sum NaN, not an integer
@@ -292,7 +296,6 @@ __global__ void __launch_bounds__(kMaxThreads, Form<Real>::kBlocks) readout_fixe
                     } else {
                         re48 += SplitSum::fixed(first(sum.a), first(sum.b), first(sum.c));
                         im48 += SplitSum::fixed(second(sum.a), second(sum.b), second(sum.c));
-                        ++tiles48;
                     }
                 }
             } else {
@@ -303,7 +306,7 @@ __global__ void __launch_bounds__(kMaxThreads, Form<Real>::kBlocks) readout_fixe
         }
     }
     if constexpr (!kF64)
-        if (tiles48) flush();
+        if (ea48) flush();
     // over a combination's threads, in order
     __syncthreads();
     double *const red = (double *)smem;  // [nsub][cpb][2]: at most 8 KiB, where the table was
@@ -312,7 +315,7 @@ __global__ void __launch_bounds__(kMaxThreads, Form<Real>::kBlocks) readout_fixe
         red[2 * threadIdx.x + 1] = im;
     }
     __syncthreads();
-    double *const out = p.part + (int64_t)blockIdx.y * (p.n_combo + 1) * 2;
+    double *const out = p.part + chunk * (p.n_combo + 1) * 2;
     if (active && sub == 0) {
         for (int k = 1; k < p.nsub; ++k) {
             re += red[2 * (k * p.cpb + mine)];
@@ -387,11 +390,12 @@ chunk_sums_kernel(const double *part, int32_t n_chunks, int32_t n_combo, double 
 // threads, at most kMaxPairs pairs), threads a combination, and walkers a
 // block -- a whole wave of the blocks that are resident for few groups, four
 // waves (whose last is less empty) for many, whole tiles, at most max_chunks.  The
-// plain form adds a chunk's tiles one after another in FP64, which is off by n / 8
-// sqrt(W) for chunks of n walkers where sums over 4096 single walkers are off by
-// 4096 / sqrt(W): as many times the chunks, where one would be longer than half of
-// 8 x 4096 (1e6 walkers x 131 072 combinations: 5.6 2^-53 off in the mean square with
-// 4 chunks, 0.88 with sums over 4096, 0.65 with 64; the same time).
+// plain form's sums and the sum of alpha add a chunk's tiles one after another in
+// FP64, which is off by n / 8 sqrt(W) for chunks of n walkers where sums over 4096
+// single walkers are off by 4096 / sqrt(W): as many times the chunks, where one would
+// be longer than half of 8 x 4096 (plain form, 1e6 walkers x 131 072 combinations:
+// 5.6 2^-53 off in the mean square with 4 chunks, 0.88 with sums over 4096, 0.65 with
+// 64; the same time).
 template <typename Real>
 ReadoutPlan<Real> readout_plan(int64_t W, int32_t S, int32_t n_dirs, int32_t n_b, int64_t max_chunks)
 {
@@ -411,7 +415,7 @@ ReadoutPlan<Real> readout_plan(int64_t W, int32_t S, int32_t n_dirs, int32_t n_b
     p.pitch = (int32_t)std::min<int64_t>((int64_t)S * n_dirs, (p.cpb - 1) / n_b + 2) | 1;  // odd: no bank conflicts
     constexpr int64_t kWave = Form<Real>::kBlocks * 152;
     int64_t chunks = std::max<int64_t>(1, (groups <= 8 ? kWave : 4 * kWave) / groups);
-    if constexpr (sizeof(Real) == 8) chunks *= (W + chunks * kMostWalkers - 1) / (chunks * kMostWalkers);
+    chunks *= (W + chunks * kMostWalkers - 1) / (chunks * kMostWalkers);
     chunks = std::min(std::min(chunks, (W + kTile - 1) / kTile), max_chunks);
     p.per = ((W + chunks - 1) / chunks + kTile - 1) / kTile * kTile;
     p.n_chunks = (int32_t)((W + p.per - 1) / p.per);
@@ -421,6 +425,9 @@ ReadoutPlan<Real> readout_plan(int64_t W, int32_t S, int32_t n_dirs, int32_t n_b
 template <typename Real>
 cudaError_t launch_readout(const ReadoutPlan<Real> &p, cudaStream_t stream)
 {
+    // the FP32 form's integer sums have room for chunks of this length
+    static_assert((kMostWalkers / kTile) * (64ll << 48) <= 1ll << 62, "integer sums of a chunk");
+    if (sizeof(Real) == 4 && p.per > kMostWalkers) return cudaErrorInvalidValue;
     // the largest any plan needs, so that host threads do not set different limits;
     // per context, and cheap: asked for at every launch
     constexpr size_t kMost = smem_bytes<Real>(kMaxShapes, kMaxPairs | 1);
@@ -428,8 +435,9 @@ cudaError_t launch_readout(const ReadoutPlan<Real> &p, cudaStream_t stream)
     const cudaError_t e =
         cudaFuncSetAttribute(readout_fixed_kernel<Real>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kMost);
     if (e != cudaSuccess) return e;
-    readout_fixed_kernel<Real><<<dim3((unsigned)p.groups, (unsigned)p.n_chunks), p.threads,
-                                 smem_bytes<Real>(p.S, p.pitch), stream>>>(p);
+    const unsigned ny = (unsigned)std::min(p.n_chunks, 32768);
+    const dim3 grid((unsigned)p.groups, ny, ((unsigned)p.n_chunks + ny - 1) / ny);
+    readout_fixed_kernel<Real><<<grid, p.threads, smem_bytes<Real>(p.S, p.pitch), stream>>>(p);
     return cudaGetLastError();
 }
 
