@@ -233,19 +233,18 @@ __global__ void trig_table_kernel(double *trig)
     trig[2 * j + 1] = sn;
 }
 
-// Per step: the weights dt G_{s,k} (rows of `pitch`, zeros beyond the last
-// step) and the step flags.
+// Per step: the weights dt G_{s,k} and the step flags.
 // Sets bit 1 of warn where a weight is out of the unchecked arithmetic's range.
-__global__ void step_tables_kernel(int64_t N, int64_t pitch, int32_t S, double dt, const double *G, double *wG64,
-                                   float *wG32, uint8_t *flags, int32_t *warn)
+__global__ void step_tables_kernel(int64_t N, int32_t S, double dt, const double *G, double *wG64, float *wG32,
+                                   uint8_t *flags, int32_t *warn)
 {
     const int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;  // 0-based step index
-    if (k >= pitch) return;
+    if (k >= N) return;
     uint8_t f = 0;
     for (int s = 0; s < S; ++s) {
-        const double w = k < N ? dt * G[(int64_t)s * N + k] : 0.0;
-        wG64[(int64_t)s * pitch + k] = w;
-        wG32[(int64_t)s * pitch + k] = (float)w;
+        const double w = dt * G[(int64_t)s * N + k];
+        wG64[(int64_t)s * N + k] = w;
+        wG32[(int64_t)s * N + k] = (float)w;
         if (w != 0.0) f = 1u;
         if (!(w == 0.0 || (fabs(w) >= 0x1p-400 && fabs(w) <= 0x1p400))) atomicOr(warn, 2);
     }
@@ -800,11 +799,10 @@ static rms_status set_sequence_impl(rms_substrate *sub, const rms_sequence_desc 
     RMS_CUDA(cudaMallocAsync((void **)&q->d_dtR32, sizeof(float) * 3 * L, st));
     RMS_CUDA(cudaMallocAsync((void **)&q->d_T, sizeof(uint32_t) * (size_t)L * L, st));
     if (sub->d_rho) RMS_CUDA(cudaMallocAsync((void **)&q->d_Tmt, sizeof(uint32_t) * (size_t)L * L, st));
-    q->pitch = (N / 8 + 2) * 8;  // whole vectors of 8 steps, at least one step beyond the last
-    const size_t nG = (size_t)S * q->pitch;
+    const size_t nG = (size_t)S * (N ? N : 1);
     RMS_CUDA(cudaMallocAsync((void **)&q->d_wG64, sizeof(double) * nG, st));
     RMS_CUDA(cudaMallocAsync((void **)&q->d_wG32, sizeof(float) * nG, st));
-    RMS_CUDA(cudaMallocAsync((void **)&q->d_flags, (size_t)q->pitch, st));
+    RMS_CUDA(cudaMallocAsync((void **)&q->d_flags, (size_t)(N ? N : 1), st));
     const std::vector<int32_t> rec32(q->rec_steps.begin(), q->rec_steps.end());  // n_steps <= 2e9
     RMS_TRY(upload(&q->d_rec_step, rec32.data(), rec32.size(), st));
     if (d->mode) {
@@ -836,8 +834,9 @@ static rms_status set_sequence_impl(rms_substrate *sub, const rms_sequence_desc 
         host_pair_tables(sub, d->dt_ms, hostT, host_warn);
         RMS_CUDA(cudaMemcpyAsync(q->d_T, hostT.data(), sizeof(uint32_t) * hostT.size(), cudaMemcpyHostToDevice, st));
     }
-    step_tables_kernel<<<(unsigned)((q->pitch + 255) / 256), 256, 0, st>>>(N, q->pitch, S, d->dt_ms, d_G, q->d_wG64,
-                                                                            q->d_wG32, q->d_flags, d_warn);
+    if (N > 0)
+        step_tables_kernel<<<(unsigned)((N + 255) / 256), 256, 0, st>>>(N, S, d->dt_ms, d_G, q->d_wG64, q->d_wG32,
+                                                                         q->d_flags, d_warn);
     bvalue_kernel<<<(unsigned)std::max(S, 1), kBvThreads, 0, st>>>(N, S, d->dt_ms, d_G, d->n_b, q->d_b, q->d_bs,
                                                                     q->d_q);
     RMS_CUDA(cudaGetLastError());
@@ -939,18 +938,17 @@ ReqDesc<Real> rms::run_desc(rms_run_handle *r)
                    sub->periodic[0] | sub->periodic[1] << 1 | sub->periodic[2] << 2, sub->voxel_um,
                    (float)sub->voxel_um};
     if constexpr (std::is_same<Real, float>::value) {
-        d.t = Tables<float>{q->d_s32, q->d_dtR32, q->d_T, q->d_Tmt, sub->L, q->d_wG32, q->pitch, q->d_flags,
+        d.t = Tables<float>{q->d_s32, q->d_dtR32, q->d_T, q->d_Tmt, sub->L, q->d_wG32, q->n_steps, q->d_flags,
                             q->d_rec_step, q->d_mode, q->any_relax, q->d_trig};
         d.st = r->st32;
     } else {
-        d.t = Tables<double>{q->d_s64, q->d_dtR64, q->d_T, q->d_Tmt, sub->L, q->d_wG64, q->pitch, q->d_flags,
+        d.t = Tables<double>{q->d_s64, q->d_dtR64, q->d_T, q->d_Tmt, sub->L, q->d_wG64, q->n_steps, q->d_flags,
                              q->d_rec_step, q->d_mode, q->any_relax, q->d_trig};
         d.st = r->st64;
     }
     d.ctl.seed = r->seed;
     d.ctl.w_begin = r->w_begin;
     d.ctl.n_walkers = r->W;
-    d.ctl.n_steps = q->n_steps;
     d.ctl.n_shapes = q->S;
     d.ctl.n_rec = q->n_rec;
     d.ctl.status = r->d_status;

@@ -186,8 +186,8 @@ struct Tables {
     const uint32_t *T;      // [from][to] Bernoulli thresholds
     const uint32_t *Tmt;    // [from][to] saturation thresholds (MT), or nullptr
     int32_t n_labels;
-    const Real *wG;         // [shape][pitch]: dt * G of each step, zeros beyond the last
-    int64_t pitch;
+    const Real *wG;         // [shape][n_steps]: dt * G of each step
+    int64_t n_steps;
     const uint8_t *flags;   // [step]: 1 where some shape's G != 0
     const int32_t *rec_step;  // [n_rec] recording steps
     const uint8_t *mode;    // [step] relaxation mode (or nullptr = 0)
@@ -199,7 +199,6 @@ struct RunCtl {
     uint64_t seed;
     int64_t w_begin;
     int64_t n_walkers;
-    int64_t n_steps;
     int32_t n_shapes;
     int32_t n_rec;
     int32_t *status;                // device error bits

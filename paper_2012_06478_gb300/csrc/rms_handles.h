@@ -61,7 +61,6 @@ struct rms_sequence {
     uint32_t *d_Tmt = nullptr;  // saturation thresholds (nullptr: no absorbing membrane)
     uint8_t *d_flags = nullptr, *d_mode = nullptr;
     int32_t *d_rec_step = nullptr;
-    int64_t pitch = 0;  // row pitch of d_wG64 and d_wG32
     double *d_dirs = nullptr, *d_b = nullptr, *d_bs = nullptr, *d_q = nullptr;
     double *d_trig = nullptr;  // azimuth table (FP64 form)
     // Cancel flags of this sequence's runs: mapped host memory taken at the first

@@ -18,8 +18,8 @@
 // What bounds it: the FP32 step issues (332 warp-instructions per warp-step on
 // 200x200x400 axons, issue slots 77 % used, ALU pipe 64 %).  Deciding the
 // events from face bits instead of a label gather with wrapped coordinates,
-// with selects in place of branches, the step's tables and weights read ahead
-// and nothing done for relaxation when no label relaxes took 1e6 walkers x
+// with selects in place of branches, the step's weight asked for before the
+// walk and nothing done for relaxation when no label relaxes took 1e6 walkers x
 // 2000 steps from 27.4 ms (428 warp-instructions) to 21.8 ms; packed phase sums
 // and octants without selects took the call of 10 000 steps from 112.6 ms to
 // 108.4; the same bits.  The plain form's step uses the ALU, the integer
@@ -984,7 +984,7 @@ __device__ __forceinline__ void walk_block(const Geometry &g, const Tables<Real>
         }
         // ---- phase (Eq. 7, right end point of each step)
         if (graded) {
-            const auto weight = [&](int s) { return NS == 1 ? wg : __ldg(t.wG + (int64_t)s * t.pitch + (k - 1)); };
+            const auto weight = [&](int s) { return NS == 1 ? wg : __ldg(t.wG + (int64_t)s * t.n_steps + (k - 1)); };
             if constexpr (kF64) {
 #pragma unroll 1
                 for (int r = 0; r < 3; ++r) {
@@ -1165,22 +1165,23 @@ cudaError_t launch_walk(int n_shapes, bool hash, dim3 grid, cudaStream_t stream,
 // three and six shapes where they pay: the FP32 form's elastic collision
 #define RMS_LAUNCH_NS(HASHV, RELAXV)                                                  \
     do {                                                                              \
-        constexpr bool kPlain = std::is_same<Real, double>::value;                    \
-        constexpr bool kMore = !kPlain && IM == kInteractEC && !MT && !HASHV;         \
-        if (n_shapes <= 1)                                                            \
+        constexpr bool kMore = IM == kInteractEC && !MT && !HASHV;                    \
+        if (n_shapes <= 1) {                                                          \
             RMS_LAUNCH(1, HASHV, RELAXV);                                             \
-        else if (kPlain)                                                              \
+        } else if constexpr (std::is_same<Real, double>::value) {                     \
             RMS_LAUNCH(8, HASHV, RELAXV);                                             \
-        else if (n_shapes <= 2)                                                       \
-            RMS_LAUNCH(kPlain ? 8 : 2, HASHV, RELAXV);                                             \
-        else if (kMore && n_shapes <= 3)                                              \
-            RMS_LAUNCH(kMore ? 3 : 8, HASHV, RELAXV);                                 \
-        else if (n_shapes <= 4)                                                       \
-            RMS_LAUNCH(kPlain ? 8 : 4, HASHV, RELAXV);                                             \
-        else if (kMore && n_shapes <= 6)                                              \
-            RMS_LAUNCH(kMore ? 6 : 8, HASHV, RELAXV);                                 \
-        else                                                                          \
-            RMS_LAUNCH(8, HASHV, RELAXV);                                             \
+        } else {                                                                      \
+            if (n_shapes <= 2)                                                        \
+                RMS_LAUNCH(2, HASHV, RELAXV);                                         \
+            else if (n_shapes <= (kMore ? 3 : 0))                                     \
+                RMS_LAUNCH(kMore ? 3 : 4, HASHV, RELAXV);                             \
+            else if (n_shapes <= 4)                                                   \
+                RMS_LAUNCH(4, HASHV, RELAXV);                                         \
+            else if (n_shapes <= (kMore ? 6 : 0))                                     \
+                RMS_LAUNCH(kMore ? 6 : 8, HASHV, RELAXV);                             \
+            else                                                                      \
+                RMS_LAUNCH(8, HASHV, RELAXV);                                         \
+        }                                                                             \
     } while (0)
     if (hash)
         RMS_LAUNCH_NS(true, 2);

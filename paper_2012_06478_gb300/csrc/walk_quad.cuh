@@ -184,7 +184,7 @@ walk_quad_kernel(Geometry g, Tables<double> t, WalkerState<double> st, RunCtl ct
 #pragma unroll
             for (int s = 0; s < NS; ++s)
                 if (s < ctl.n_shapes)
-                    ph[s] = ph[s] + times_any<SANE>(NS == 1 ? wg : __ldg(t.wG + (int64_t)s * t.pitch + (k - 1)), dx);
+                    ph[s] = ph[s] + times_any<SANE>(NS == 1 ? wg : __ldg(t.wG + (int64_t)s * t.n_steps + (k - 1)), dx);
         }
         // ---- displacement moments: the first warp sums the block's 32 walkers as
         //      the one-thread kernel's warp does
