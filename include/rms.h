@@ -429,7 +429,15 @@ rms_status rms_philox4x32_10(const uint32_t *ctr, const uint32_t *key, int64_t n
 
 /* The same read-out as rms_run's in the plain FP64 form (S = sum alpha
  * e^{-i phi} / sum alpha, phi = q g.Phi_s, q = sqrt(b / b_s), alpha =
- * exp(-A), every term within 2^-52 of alpha's largest) over walker data the caller holds.  Every pointer is a DEVICE pointer of the current device:
+ * exp(-A)) over walker data the caller holds.  Walkers are taken 64 at a time;
+ * with a the largest alpha and P the largest |phi| (rad) of a walker's 64, the
+ * real and imaginary parts of its term alpha e^{-i phi} are within
+ * a (2^-51.8 + 2^-55 P) of their values for the phi that FP64 gives (dot product
+ * and q rounded: within 5 2^-53 of q sum |g_i Phi_i|); the bound is relative to
+ * a, not to the walker's own alpha.
+ * FP64 sincos and sums instead for fewer than 256 walkers and for 64 with P
+ * below 2^-6, above 2^20 or not finite, or with a zero or not finite.
+ * Every pointer is a DEVICE pointer of the current device:
  *   phase     : n_walkers*n_shapes*3 doubles, row-major (walker, shape, axis),
  *               the layout rms_read_walkers returns
  *   A         : n_walkers doubles, exponent of Eq. 5

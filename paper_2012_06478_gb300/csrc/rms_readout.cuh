@@ -8,10 +8,11 @@
 // of the FP64 operations.
 //
 // Precision, against sincos and FP64 sums: the phase is within 2^-57 of the
-// largest |phase| of 64 walkers (a double's last place is 2^-53 of it), the
-// term within about 2^-54 of the largest alpha, its rounding is not biased and
-// the sum over 64 walkers is exact, so a signal is nearer to its exact value
-// than FP64 sums over 4096 walkers bring it.  Phases too small (below 2^-6
+// largest |phase| P of 64 walkers (a double's last place is 2^-53 of it), the
+// term's parts within 2^-51.8 + 2^-55 P of their largest alpha (2^-55 in the mean
+// square at |phase| < 1), its rounding is not biased and the sum over 64 walkers is
+// exact, so a signal is nearer to its exact value than FP64 sums over 4096
+// walkers bring it.  Phases too small (below 2^-6
 // rad), too large (above 2^20 rad) or not finite, and alphas that are not
 // finite or all zero, take sincos in FP64 (rms_readout.cu).
 //
