@@ -12,6 +12,7 @@ import numpy as np
 import pytest
 
 from conftest import make_workload
+from test_gpu_readout_sizes import _exact, _readout
 
 pytestmark = pytest.mark.gpu
 
@@ -49,3 +50,24 @@ def test_sums_over_many_walkers():
     re, im = (share[:, None, None] * np.cos(phi)).sum(0), -(share[:, None, None] * np.sin(phi)).sum(0)
     off = np.sqrt(float(((S[0][:, some].real - re) ** 2 + (S[0][:, some].imag - im) ** 2).mean()))
     assert off <= 2 * 2.0 ** -53, off * 2.0 ** 53
+
+
+@pytest.mark.parametrize("W,S,nd,nb", [(256, 1, 3, 2), (257, 1, 30, 11), (1000, 8, 5, 1), (3001, 1, 64, 9),
+                                       (4097, 1, 130, 1), (20001, 2, 3, 4), (9999, 3, 70, 5)])
+def test_groups_and_remainders_of_ordinary_walkers(W, S, nd, nb):
+    """Several groups of combinations, part tiles and part chunks, with phases of a few
+    radians alone: within a term's bound, the dot product's and three roundings."""
+    rng = np.random.default_rng([W, nd])
+    phase = rng.normal(size=(W, S, 3)) * 0.5
+    A = rng.uniform(0.0, 3.0, size=W)
+    dirs = rng.normal(size=(nd, 3))
+    dirs /= np.linalg.norm(dirs, axis=1, keepdims=True)
+    bs = rng.uniform(0.7, 1.4, size=S)
+    b = np.linspace(0.5, 8.0, nb)
+    got, asum = _readout(phase, A, bs, dirs, b)
+    want, asum_w = _exact(phase, A, bs, dirs, b)
+    P = np.sqrt(b.max() / bs.min()) * (np.abs(phase) @ np.abs(dirs).T).max()
+    # the terms' bound is relative to alphas of 1 at most, the signal to their mean
+    tol = (2.0 ** -51.8 + 2.0 ** -55 * P) / np.exp(-A).mean() + 5 * 2.0 ** -53 * P + 3 * 2.0 ** -53
+    assert max(np.abs((got - want).real).max(), np.abs((got - want).imag).max()) <= tol
+    assert abs(asum - asum_w) <= 1e-14 * asum_w
