@@ -2,12 +2,13 @@
 // (paper_2012_06478_gb300/csrc/soft_fp64.cuh) as the GPU computes them, against
 // the GPU's own IEEE operations: products with exact ties, with every carry of
 // the rounding (all-ones kept parts, kept parts of zeros), of random and of
-// extreme significands; quotients and roots a unit around a rounding midpoint.
-// Prints the cases compared and the mismatches of each; exit status 1 on a
+// extreme significands; quotients and roots a unit around a rounding midpoint; and
+// the operands of soft_fp64_edges.h.  Prints the cases compared and the mismatches of each; exit status 1 on a
 // mismatch.
 #include <cstdio>
 
 #include "../paper_2012_06478_gb300/csrc/soft_fp64.cuh"
+#include "soft_fp64_edges.h"
 
 using namespace rms::sfp;
 
@@ -87,11 +88,30 @@ __global__ void check(long cases, Count *n)
     }
 }
 
+__global__ void check_edges(const EdgeCase *c, long cases, Count *n)
+{
+    const long i = blockIdx.x * (long)blockDim.x + threadIdx.x;
+    if (i >= cases) return;
+    const double a = c[i].a, b = c[i].b;
+    if (c[i].op == 0)
+        compare(n, 0, mul_normal(a, b), __dmul_rn(a, b));
+    else if (c[i].op == 1)
+        compare(n, 1, div_normal(a, b), __ddiv_rn(a, b));
+    else
+        compare(n, 2, sqrt_normal(a), __dsqrt_rn(a));
+}
+
 int main()
 {
     Count *n = nullptr, h{};
     if (cudaMalloc((void **)&n, sizeof *n) != cudaSuccess || cudaMemset(n, 0, sizeof *n) != cudaSuccess) return 2;
     check<<<608, 128>>>(2000000, n);
+    const std::vector<EdgeCase> e = edges::cases(200000, 4);
+    EdgeCase *d = nullptr;
+    if (cudaMalloc((void **)&d, sizeof(EdgeCase) * e.size()) != cudaSuccess ||
+        cudaMemcpy(d, e.data(), sizeof(EdgeCase) * e.size(), cudaMemcpyHostToDevice) != cudaSuccess)
+        return 2;
+    check_edges<<<(unsigned)((e.size() + 127) / 128), 128>>>(d, (long)e.size(), n);
     if (cudaGetLastError() != cudaSuccess || cudaMemcpy(&h, n, sizeof h, cudaMemcpyDeviceToHost) != cudaSuccess) return 2;
     for (int k = 0; k < 3; ++k) std::printf("%llu %llu\n", h.tested[k], h.bad[k]);
     return h.bad[0] || h.bad[1] || h.bad[2] ? 1 : 0;
