@@ -20,9 +20,12 @@ __device__ const fix::Octant g_octant = fix::octant_table();
 
 constexpr int kTile = 64;         // walkers staged at a time: their exact sums fit 64 bits
 constexpr int kMaxThreads = 512;
+constexpr int kFewThreads = 128;  // below kMinWalkers
 constexpr int kMaxPairs = 130;    // (shape, direction) pairs of one block's combinations, at most
 constexpr int64_t kMostWalkers = 16384;  // of a chunk, but for a limit on chunks
 constexpr int kMinWalkers = 256;  // fewer: floating-point terms (their roundings are not averaged out)
+
+constexpr size_t kSums = sizeof(double) * 2 * kMaxThreads;  // the last sums, where the table was
 
 // The forms' staged numbers: the plain form's terms are integers; the FP32
 // form's single precision (phi, sincosf and the product with alpha), with sums
@@ -34,14 +37,14 @@ struct Form<double> {
     using Alpha = fix::Words;
     using Phase = int64_t;
     static constexpr int kBlocks = 2;  // resident blocks per SM
-    static constexpr size_t kTable = sizeof(fix::Angle) * fix::kAngles;
+    static constexpr size_t kTable = sizeof(fix::Angle) * fix::kAngles;  // none below kMinWalkers
 };
 template <>
 struct Form<float> {
     using Alpha = float;
     using Phase = float;
     static constexpr int kBlocks = 3;
-    static constexpr size_t kTable = sizeof(double) * 2 * kMaxThreads;  // the last sums' place
+    static constexpr size_t kTable = kSums;
 };
 
 // alpha given in 58 bits of a power of two
@@ -101,11 +104,17 @@ __device__ __noinline__ double2 plain_sums(const float *v, int K, const double *
 }
 
 template <typename Real>
-constexpr size_t smem_bytes(int S, int pitch)
+__host__ __device__ constexpr size_t table_bytes(int64_t W)
+{
+    return W >= kMinWalkers ? Form<Real>::kTable : kSums;
+}
+
+template <typename Real>
+constexpr size_t smem_bytes(int64_t W, int S, int pitch)
 {
     using F = Form<Real>;
     const int rows = (sizeof(Real) == 8 ? 1 : 2) * (3 * S + 1);
-    return F::kTable + sizeof(double) * kTile + sizeof(Real) * 2 * rows * kTile + sizeof(typename F::Alpha) * kTile +
+    return table_bytes<Real>(W) + sizeof(double) * kTile + sizeof(Real) * 2 * rows * kTile + sizeof(typename F::Alpha) * kTile +
            sizeof(typename F::Phase) * kTile * pitch + sizeof(int) * pitch;
 }
 
@@ -130,7 +139,7 @@ __global__ void __launch_bounds__(kMaxThreads, Form<Real>::kBlocks) readout_fixe
     auto *const table = (fix::Angle *)smem;  // plain form
     // staged numbers of a walker: its phases and A (FP32 form: phases, compensations, A and A's)
     const int K = 3 * p.S, KA = kF64 ? K : 2 * K, rows = kF64 ? K + 1 : 2 * K + 2;
-    double *const alD = (double *)(smem + F::kTable);                 // alpha of the tile
+    double *const alD = (double *)(smem + table_bytes<Real>(p.W));    // alpha of the tile
     Real *const raw = (Real *)(alD + kTile);                          // [2][rows][kTile]
     auto *const alF = (typename F::Alpha *)(raw + 2 * rows * kTile);  // over a power of two above the largest
     auto *const X = (typename F::Phase *)(alF + kTile);               // [kTile][pitch]
@@ -138,7 +147,7 @@ __global__ void __launch_bounds__(kMaxThreads, Form<Real>::kBlocks) readout_fixe
     __shared__ double s_asum;
     __shared__ int s_ea;  // exponent of the tile's largest alpha; 0: floating-point terms
 
-    if constexpr (kF64)
+    if (kF64 && p.W >= kMinWalkers)  // fewer: no term takes it
         for (int k = threadIdx.x; k < fix::kAngles; k += blockDim.x) table[k] = fix::angle_of(g_octant, k);
 
     const int64_t chunk = (int64_t)blockIdx.z * gridDim.y + blockIdx.y;
@@ -160,11 +169,13 @@ __global__ void __launch_bounds__(kMaxThreads, Form<Real>::kBlocks) readout_fixe
         pair -= pair0;
     }
     const int64_t Q = fix::turns_of(q);
+    // the pairs' g.Phi: of few walkers only what b = 0 asks for, whether it is finite
+    const bool pairs = __syncthreads_or(active && q == 0.0) || p.W >= kMinWalkers;
 
     const int64_t w0 = chunk * p.per, w1 = min(p.W, w0 + p.per);
     const auto stage = [&](int64_t base, Real *to) {  // asynchronous copy of a tile's walkers
         const int nt = (int)min((int64_t)kTile, w1 - base);
-        for (int e = threadIdx.x; e < rows * kTile; e += blockDim.x) {
+        for (int e = threadIdx.x; e < rows * (p.sw == 1 ? kTile : nt); e += blockDim.x) {
             // neighbouring threads take neighbouring numbers of memory
             const int j = p.sw == 1 ? e % kTile : e / rows, k = p.sw == 1 ? e / kTile : e % rows;
             if (j >= nt) continue;
@@ -200,7 +211,7 @@ __global__ void __launch_bounds__(kMaxThreads, Form<Real>::kBlocks) readout_fixe
         __syncthreads();  // the tile has come, and the sums of the one before are done
         if (base + kTile < w1) stage(base + kTile, raw + (at ^ 1) * rows * kTile);
         // a warp each: alpha, and g.Phi of one pair at a time
-        for (int t = warp; t <= n_pairs; t += n_warps) {
+        for (int t = pairs ? warp : n_pairs + warp; t <= n_pairs; t += n_warps) {
             if (t == n_pairs) {
                 double x[2];
                 for (int h = 0; h < 2; ++h) {
@@ -341,7 +352,7 @@ __device__ __forceinline__ void neumaier(double &sum, double &comp, double x)
 }
 
 // Sums over walker chunks in a fixed order.  A block has 32 combinations; its
-// eight warps take every eighth chunk each (one thread over all chunks took
+// warps, eight at most, take every eighth chunk each (one thread over all chunks took
 // 233 us for 2442 chunks x 513 combinations, a chain of dependent FP64
 // additions; eight at once, and fewer chunks, 48 us).  NORM: the last column,
 // the sum of alpha, divides the others (split real and imaginary parts,
@@ -353,12 +364,12 @@ __global__ void __launch_bounds__(32 * kSumWarps)
 chunk_sums_kernel(const double *part, int32_t n_chunks, int32_t n_combo, double *out_re, double *out_im, double *alpha)
 {
     __shared__ double sh[kSumWarps][6][32];
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, warps = blockDim.x >> 5;
     const int64_t combo = (int64_t)blockIdx.x * 32 + lane;
     const bool active = NORM ? combo < n_combo : combo <= n_combo;
     double v[6] = {};  // sum and compensation of the real and imaginary parts and of alpha
     if (active) {
-        for (int64_t k = warp; k < n_chunks; k += kSumWarps) {
+        for (int64_t k = warp; k < n_chunks; k += warps) {
             const double *row = part + k * (n_combo + 1) * 2;
             neumaier(v[0], v[1], row[2 * combo]);
             neumaier(v[2], v[3], row[2 * combo + 1]);
@@ -368,8 +379,8 @@ chunk_sums_kernel(const double *part, int32_t n_chunks, int32_t n_combo, double 
     }
     __syncthreads();
     if (warp != 0 || !active) return;
-    for (int k = 1; k < kSumWarps; ++k)
-        for (int i = 0; i < 6; i += 2) {
+    for (int k = 1; k < warps; ++k)
+        for (int i = 0; i < (NORM ? 6 : 4); i += 2) {
             neumaier(v[i], v[i + 1], sh[k][i][lane]);
             v[i + 1] += sh[k][i + 1][lane];
         }
@@ -389,7 +400,10 @@ chunk_sums_kernel(const double *part, int32_t n_chunks, int32_t n_combo, double 
 // How the read-out splits: combinations a block (one group when they fit its
 // threads, at most kMaxPairs pairs), threads a combination, and walkers a
 // block -- a whole wave of the blocks that are resident for few groups, four
-// waves (whose last is less empty) for many, whole tiles, at most max_chunks.  The
+// waves (whose last is less empty) for many, whole tiles, at most max_chunks.
+// Below kMinWalkers a thread's chain of sincos takes the time: blocks of kFewThreads,
+// of as few combinations as leave two blocks an SM (100 walkers x 330 combinations 32 us
+// against 249 in one block of 352 threads a tile, 1 x 6 21.9 against 34.6).  The
 // plain form's sums and the sum of alpha add a chunk's tiles one after another in
 // FP64, which is off by n / 8 sqrt(W) for chunks of n walkers where sums over 4096
 // single walkers are off by 4096 / sqrt(W): as many times the chunks, where one would
@@ -405,18 +419,22 @@ ReadoutPlan<Real> readout_plan(int64_t W, int32_t S, int32_t n_dirs, int32_t n_b
     p.n_dirs = n_dirs;
     p.n_b = n_b;
     p.n_combo = S * n_dirs * n_b;
-    const int64_t most = std::min<int64_t>(kMaxThreads, (int64_t)(kMaxPairs - 2) * n_b);
+    const int64_t tiles = (W + kTile - 1) / kTile;
+    const bool few = W < kMinWalkers;
+    const int64_t threads = few ? kFewThreads : kMaxThreads, lanes = std::min<int64_t>(kTile, W);
+    int64_t most = std::min<int64_t>(threads, (int64_t)(kMaxPairs - 2) * n_b);
+    if (few) most = std::min(most, std::max(threads / lanes, p.n_combo * tiles / (2 * 152)));
     int64_t groups = (p.n_combo + most - 1) / most;
     p.cpb = (int32_t)((p.n_combo + groups - 1) / groups);
     groups = (p.n_combo + p.cpb - 1) / p.cpb;
-    p.nsub = std::min<int32_t>(kTile, kMaxThreads / p.cpb);
+    p.nsub = (int32_t)std::min(lanes, threads / p.cpb);
     p.threads = (p.cpb * p.nsub + 31) / 32 * 32;
     p.groups = (int32_t)groups;
     p.pitch = (int32_t)std::min<int64_t>((int64_t)S * n_dirs, (p.cpb - 1) / n_b + 2) | 1;  // odd: no bank conflicts
     constexpr int64_t kWave = Form<Real>::kBlocks * 152;
     int64_t chunks = std::max<int64_t>(1, (groups <= 8 ? kWave : 4 * kWave) / groups);
     chunks *= (W + chunks * kMostWalkers - 1) / (chunks * kMostWalkers);
-    chunks = std::min(std::min(chunks, (W + kTile - 1) / kTile), max_chunks);
+    chunks = std::min(std::min(chunks, tiles), max_chunks);
     p.per = ((W + chunks - 1) / chunks + kTile - 1) / kTile * kTile;
     p.n_chunks = (int32_t)((W + p.per - 1) / p.per);
     return p;
@@ -430,14 +448,14 @@ cudaError_t launch_readout(const ReadoutPlan<Real> &p, cudaStream_t stream)
     if (sizeof(Real) == 4 && p.per > kMostWalkers) return cudaErrorInvalidValue;
     // the largest any plan needs, so that host threads do not set different limits;
     // per context, and cheap: asked for at every launch
-    constexpr size_t kMost = smem_bytes<Real>(kMaxShapes, kMaxPairs | 1);
+    constexpr size_t kMost = smem_bytes<Real>(kMinWalkers, kMaxShapes, kMaxPairs | 1);
     static_assert(kMost <= 227 * 1024, "shared memory of a block");
     const cudaError_t e =
         cudaFuncSetAttribute(readout_fixed_kernel<Real>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kMost);
     if (e != cudaSuccess) return e;
     const unsigned ny = (unsigned)std::min(p.n_chunks, 32768);
     const dim3 grid((unsigned)p.groups, ny, ((unsigned)p.n_chunks + ny - 1) / ny);
-    readout_fixed_kernel<Real><<<grid, p.threads, smem_bytes<Real>(p.S, p.pitch), stream>>>(p);
+    readout_fixed_kernel<Real><<<grid, p.threads, smem_bytes<Real>(p.W, p.S, p.pitch), stream>>>(p);
     return cudaGetLastError();
 }
 
@@ -449,14 +467,14 @@ template cudaError_t launch_readout<float>(const ReadoutPlan<float> &, cudaStrea
 cudaError_t launch_chunk_sums(const double *part, int32_t n_chunks, int32_t n_combo, double *out, cudaStream_t stream)
 {
     chunk_sums_kernel<false>
-        <<<(unsigned)(n_combo / 32 + 1), 32 * kSumWarps, 0, stream>>>(part, n_chunks, n_combo, out, nullptr, nullptr);
+        <<<(unsigned)(n_combo / 32 + 1), 32 * std::min(kSumWarps, n_chunks), 0, stream>>>(part, n_chunks, n_combo, out, nullptr, nullptr);
     return cudaGetLastError();
 }
 
 cudaError_t launch_chunk_sums_normalised(const double *part, int32_t n_chunks, int32_t n_combo, double *S_re,
                                          double *S_im, double *alpha_sum, cudaStream_t stream)
 {
-    chunk_sums_kernel<true><<<(unsigned)((n_combo + 31) / 32), 32 * kSumWarps, 0, stream>>>(
+    chunk_sums_kernel<true><<<(unsigned)((n_combo + 31) / 32), 32 * std::min(kSumWarps, n_chunks), 0, stream>>>(
         part, n_chunks, n_combo, S_re, S_im, alpha_sum);
     return cudaGetLastError();
 }

@@ -71,3 +71,26 @@ def test_groups_and_remainders_of_ordinary_walkers(W, S, nd, nb):
     tol = (2.0 ** -51.8 + 2.0 ** -55 * P) / np.exp(-A).mean() + 5 * 2.0 ** -53 * P + 3 * 2.0 ** -53
     assert max(np.abs((got - want).real).max(), np.abs((got - want).imag).max()) <= tol
     assert abs(asum - asum_w) <= 1e-14 * asum_w
+
+
+@pytest.mark.parametrize("W,S,nd,nb", [(1, 1, 1, 1), (1, 1, 512, 1), (2, 6, 64, 11), (10, 1, 400, 25), (64, 1, 3, 2),
+                                       (65, 2, 90, 30), (100, 1, 30, 11), (200, 8, 16, 4), (255, 1, 130, 3)])
+def test_few_walkers(W, S, nd, nb):
+    """Terms in FP64, blocks of few combinations: sums of at most 64 terms a thread, 64
+    threads and 4 chunks round 132 times at most, by half a unit of a sum that is
+    the alphas' at most."""
+    rng = np.random.default_rng([W, nd, nb])
+    phase = rng.normal(size=(W, S, 3)) * 0.5
+    A = rng.uniform(0.0, 3.0, size=W)
+    dirs = rng.normal(size=(nd, 3))
+    dirs /= np.linalg.norm(dirs, axis=1, keepdims=True)
+    bs = rng.uniform(0.7, 1.4, size=S)
+    b = np.linspace(0.0, 8.0, nb) if nb > 1 else np.array([2.0])
+    got, asum = _readout(phase, A, bs, dirs, b)
+    want, asum_w = _exact(phase, A, bs, dirs, b)
+    P = np.sqrt(b.max() / bs.min()) * (np.abs(phase) @ np.abs(dirs).T).max()
+    tol = (132 + 4 + 6 * P) * 2.0 ** -53
+    assert max(np.abs((got - want).real).max(), np.abs((got - want).imag).max()) <= tol
+    assert abs(asum - asum_w) <= 136 * 2.0 ** -53 * asum_w
+    if nb > 1:
+        assert np.all(got[:, :, 0] == 1.0)
