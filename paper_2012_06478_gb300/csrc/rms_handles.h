@@ -38,7 +38,7 @@ struct rms_substrate {
     uint64_t *d_acc = nullptr;  // per label start acceptance threshold (nullptr: always)
     std::vector<uint8_t> dead;
     uint16_t *d_labels = nullptr;
-    uint8_t *d_faces = nullptr;  // face bits per voxel (rms_device.cuh)
+    uint8_t *d_faces = nullptr;  // face bits per voxel (rms_device.cuh), in d_labels' allocation
     double *d_D = nullptr, *d_T2 = nullptr, *d_T1 = nullptr, *d_kappa = nullptr, *d_rho = nullptr;
     uint8_t *d_dead = nullptr;
     int32_t *d_ok = nullptr;  // raster list of non-dead voxels (nullptr: none dead)
