@@ -166,7 +166,9 @@ typedef struct {
     void *stream;             /* cudaStream_t for the upload */
 } rms_substrate_desc;
 
-/* Upload the volume and build the per-label tables.  Errors:
+/* Upload the volume and build the per-label tables.  The substrate holds 3 bytes
+ * a voxel on the device: its label and a byte of face bits (which of the voxel's
+ * faces lead into the same label inside the volume).  Errors:
  * RMS_E_INVALID_ARG, RMS_E_OOM, RMS_E_CUDA.  The permeation and saturation
  * thresholds are built when a sequence fixes dt (rms_set_sequence). */
 rms_status rms_create_substrate(const rms_substrate_desc *desc, rms_substrate **out);

@@ -1106,11 +1106,15 @@ rms_status rms::run_walk(rms_run_handle *r, int64_t k0, int64_t k1)
     return r->precision == RMS_FP32 ? walk_impl<float>(r, k0, k1) : walk_impl<double>(r, k0, k1);
 }
 
-// Plain-form runs of at most this many walkers take four lanes to a walker.  600
-// steps of 5000, 1e4, 2e4 and 4e4 walkers in axons: 2.2, 2.4, 3.2 and 5.1 ms
-// against 4.5, 4.5, 5.2 and 6.0; with relaxation and unequal D 2.3, 2.6, 3.5 and
-// 5.8 against 4.5, 4.5, 5.2 and 6.2.  Above, the one-thread kernel's fewer
-// instructions win (3001 steps of 50 001 with relaxation: 28.5 against 30.7).
+// Plain-form runs of at most this many walkers take four lanes to a walker.  Calls of
+// 600 steps, ms, four lanes / one thread:
+//   walkers                   1e4        2.8e4      3.6e4      4.2e4      4.8e4      5.4e4
+//   axons                     1.73/2.95  2.62/3.50  3.62/3.51  3.88/4.15  4.15/4.16  4.72/4.19
+//   cells, T1, T2, unequal D  1.85/3.01  2.90/3.58  3.97/3.59  4.27/4.28  4.60/4.29  5.24/4.29
+//   axons, six waveforms, T2  2.52/4.47  4.82/5.43  5.60/5.58  6.12/6.57  6.70/6.65  8.10/6.81
+// The one-thread kernel's time goes up with every block an SM (38 912 and 58 368
+// walkers): it is level or up to 11 % ahead just below the first and 7 % at the line,
+// up to 20 % beyond it; everywhere else below the four lanes win.
 constexpr int64_t kQuadMaxWalkers = 2 * 5 * 152 * 32;
 
 // Moment partials of a block of the walk.

@@ -114,13 +114,13 @@ constexpr size_t smem_bytes(int64_t W, int S, int pitch)
 {
     using F = Form<Real>;
     const int rows = (sizeof(Real) == 8 ? 1 : 2) * (3 * S + 1);
-    return table_bytes<Real>(W) + sizeof(double) * kTile + sizeof(Real) * 2 * rows * kTile + sizeof(typename F::Alpha) * kTile +
-           sizeof(typename F::Phase) * kTile * pitch + sizeof(int) * pitch;
+    return table_bytes<Real>(W) + sizeof(double) * kTile + sizeof(Real) * 2 * rows * kTile +
+           sizeof(typename F::Alpha) * kTile + sizeof(typename F::Phase) * kTile * pitch + sizeof(int) * pitch;
 }
 
-// Grid: x a group of p.cpb combinations, y and z a chunk of p.per walkers (the groups of
-// a chunk run together and share its walkers in the L2).  A thread
-// has one combination and every p.nsub-th walker of the chunk.
+// Grid: x a group of p.cpb combinations, y and z a chunk of p.per walkers (the
+// groups of a chunk run together and share its walkers in the L2).  A thread has one
+// combination and every p.nsub-th walker of the chunk.
 //
 // What bounds it: issue, and the pipe of the 32-bit products (plain form, 1e6
 // walkers x 330 combinations: 57 % and 72 % used).  2.69 ms there, against 25.6

@@ -3,7 +3,7 @@
 // the GPU with one thread each.
 //
 // What bounds a small run: the step's dependent chain, not the arithmetic
-// units.  In the one-thread kernel a warp's step is some 3000 instructions --
+// units.  In the one-thread kernel a warp's step is some 2500 instructions --
 // the integer-ALU arithmetic of three axes, one after the other -- and with a
 // warp or two on each scheduler nothing hides their latency.  Here lane a of a
 // walker's four has axis a: its offset, displacement, face time and phases, so
@@ -14,10 +14,10 @@
 // Every operation on a walker's numbers is the one-thread kernel's, in its
 // order: the same bits.
 //
-// 600 steps of 1e4 walkers on 64^3 axons: 2.39 ms against 4.50 (one warp on each
-// of 313 schedulers before; now two on each).  Seven blocks an SM (72 registers)
-// rather than five: no difference up to 24 000 walkers, 4.08 ms against 4.53 for
-// 30 000.
+// 600 steps of 1e4 walkers on 64^3 axons, the call: 1.72 ms against 2.95 (one warp
+// on each of 313 schedulers there; here two on each).  Seven blocks an SM (72
+// registers) rather than five: 2.62 ms against 3.15 for 28 000 walkers, 2.95 against
+// 3.35 for 32 000, and 1.72 against 1.69 for 1e4.  Several waveforms have no bound.
 #pragma once
 
 #include "walk_kernel.cuh"
