@@ -76,7 +76,7 @@ typedef int rms_status;
                             first shifted right to 8 bits), so that walkers next to each other in
                             memory look up neighbouring parts of the label volume (Sec. 2.1.1: the
                             volume is the lookup table).  For volumes about the size of the L2
-                            cache or larger (measured: +23 % at 128 MB, +10 % at 256 MiB, no
+                            cache or larger (measured: +22 % at 128 MB, +5 % at 256 MiB, no
                             change at 32 MB).
                             Changes no trajectory (the random streams follow the walker id, not its
                             place in memory) and nothing rms_read_walkers / rms_read_counts return;
@@ -84,7 +84,7 @@ typedef int rms_status;
                             rounding).  Costs a second copy of the walker state and about 17 bytes
                             per walker of sort buffers.  With this flag the default launch covers
                             about 8e9 walker-steps (steps_per_launch 0), and one re-ordering of 1e7
-                            walkers takes about 1.3 % of it. */
+                            walkers takes about 1.6 % of it. */
 
 /* Particle-membrane interaction of rms_run (Sec. 2.1.2).  A face is "refused"
  * when it is impermeable (a label pair with kappa = 0, a dead label, the wall
