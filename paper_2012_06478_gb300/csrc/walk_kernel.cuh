@@ -295,8 +295,10 @@ __device__ __forceinline__ float rsqrt_normal(float x)
 
 // FP32 form of the same sampler: shorter polynomials (truncation below
 // 4e-7 on [0, pi/4]) and r from the hardware reciprocal square root (about
-// 2 ulp; (1 - z)(1 + z) > 0 since |z| < 1) -- errors of the order of the FP32
-// form's own rounding, for 2 % of its step time.
+// 2 ulp) -- errors of the order of the FP32 form's own rounding, for 2 % of its
+// step time.  For 129 of the 2^32 words z rounds to +-1, where r = 0 inf is not a
+// number: such a step (3e-8 of them) leaves x and y without a face event and its
+// clamp puts their offsets to 0.
 __device__ __forceinline__ void direction_from(uint32_t x0, uint32_t x1, const double *, float n[3])
 {
     const float z = -((float)(int32_t)(x0 ^ 0x80000000u) + 0.5f) * 0x1p-31f;
