@@ -35,7 +35,7 @@ struct Form;
 template <>
 struct Form<double> {
     using Alpha = fix::Words;
-    using Phase = int64_t;
+    using Phase = fix::Words;
     static constexpr int kBlocks = 2;  // resident blocks per SM
     static constexpr size_t kTable = sizeof(fix::Angle) * fix::kAngles;  // none below kMinWalkers
 };
@@ -123,7 +123,7 @@ constexpr size_t smem_bytes(int64_t W, int S, int pitch)
 // combination and every p.nsub-th walker of the chunk.
 //
 // What bounds it: issue, and the pipe of the 32-bit products (plain form, 1e6
-// walkers x 330 combinations: 57 % and 72 % used).  2.69 ms there, against 25.6
+// walkers x 330 combinations: 59 % and 72 % used).  2.77 ms there, against 25.6
 // with sincos and sums on the FP64 pipe; the FP32 form, whose sums on the FP64
 // pipe took 31.9 ms for 1e7 walkers x 512 combinations, 11.7 ms.
 // Tiles of 64 walkers go through shared memory twice -- the walkers' phases,
@@ -252,7 +252,7 @@ __global__ void __launch_bounds__(kMaxThreads, Form<Real>::kBlocks) readout_fixe
                     x[h] = lane + 32 * h < nt ? dot(P + 3 * ps * kTile, K, lane + 32 * h, gt) : Real(0);
                 if constexpr (kF64) {
                     const int e = top_exponent(x[0], x[1]);
-                    for (int h = 0; h < 2; ++h) X[(lane + 32 * h) * p.pitch + t] = fix::scaled(x[h], e, 62);
+                    for (int h = 0; h < 2; ++h) X[(lane + 32 * h) * p.pitch + t] = fix::words(fix::scaled(x[h], e, 62));
                     if (lane == 0) em[t] = e;
                 } else {
                     for (int h = 0; h < 2; ++h) X[(lane + 32 * h) * p.pitch + t] = x[h];
